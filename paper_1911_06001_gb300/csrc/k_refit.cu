@@ -340,6 +340,7 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
     for (int j = 0; j < P; ++j) rank += (sm.key[j] < k) ? 1 : 0;
     sm.ord[rank] = i;
     a.order[rank] = i;
+    a.sph[rank] = sm.sph[i];
   }
   __syncthreads();
   // clusters: a sphere around the member spheres, in FP32 rounded outward

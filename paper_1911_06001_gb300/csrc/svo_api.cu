@@ -69,6 +69,25 @@ constexpr unsigned long long kZeroCopyMaxRays = 1ull << 18;
 // rounded so that the second half starts 256-byte aligned.
 inline size_t stage_half_bytes(unsigned long long n) { return ((size_t)n * (32 + 16 + 4) + 255) & ~(size_t)255; }
 
+// An image trace culls whole tiles in a launch of their own from this many
+// tiles and parts (of its largest scene) on.  With fewer parts the culling
+// saved is less than the launch: its reads of the rays and about 2 us.
+// Measured per call, one launch against two:
+//   1 part, 1280x768 and shading      274 -> 288 us
+//   16 parts, 1280x768 / 1920x1080    173 -> 180 / 235 -> 227
+//   up to 24 parts, 8 views 301x199   118 -> 109
+//   63 parts, 128x128 (512 tiles)     216 -> 193
+//   up to 128 parts, 9 requests      1285 -> 1091
+//   1024 parts, 1920x1080 (grid)      731 -> 544
+constexpr unsigned long long kTileCullMin = 256;
+constexpr int kTileCullParts = 20;
+
+// Image tiles a slot of `cap` rays has entries for: an image's tiles are whole
+// 8 x 4 blocks unless its width or height leaves a remainder, so twice the
+// whole tiles hold every image of 8 x 4 pixels or more (smaller and narrower
+// ones that need more are traced in one launch).
+inline unsigned long long tile_capacity(unsigned long long cap) { return cap / 16; }
+
 constexpr size_t kCounterWords = kQueueCountWords + kMaxBatchItems / 2;
 
 // Scratch of one stream: launch counters and the FP64 re-intersection list.
@@ -81,6 +100,7 @@ struct Slot {
   uint4 *d_cand = nullptr;                   // pool of leaves stored for the FP64 pass
   unsigned long long cand_cap = 0;           // pool entries (kPoolPerRay per ray of capacity)
   uint32_t *d_off = nullptr;                 // per list slot: its first pool entry
+  TileEntry *d_tiles = nullptr;              // image tiles to trace (tile_capacity(cap) entries)
   TraceLaunch *pending = nullptr;            // launch whose FP64 pass is deferred
   char *d_stage = nullptr;                   // trace_rays_host: two halves of rays | hits | flags
   cudaStream_t pipe[3] = {nullptr, nullptr, nullptr};  // trace_rays_host: copy in, trace, copy out
@@ -124,6 +144,7 @@ struct svo_scene {
   PartAux *d_aux = nullptr;
   Cluster *d_cl = nullptr;
   int32_t *d_order = nullptr;
+  float4 *d_sph = nullptr;  // part spheres in the order of d_order
   PartStatic *d_stat = nullptr;
   int32_t *d_level_order = nullptr, *d_level_start = nullptr;
   float4 *d_bound = nullptr;
@@ -160,6 +181,8 @@ svo_status get_slot(svo_ctx *ctx, void *stream, unsigned long long need, Slot **
       CK(cudaFree(s.d_fix));
       CK(cudaFree(s.d_cand));
       CK(cudaFree(s.d_off));
+      CK(cudaFree(s.d_tiles));
+      s.d_tiles = nullptr;
       s.d_fix = nullptr;
       s.d_cand = nullptr;
       s.d_off = nullptr;
@@ -175,9 +198,11 @@ svo_status get_slot(svo_ctx *ctx, void *stream, unsigned long long need, Slot **
     cudaError_t e = cudaMalloc(&p, cap * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc(&c, ccap * sizeof(uint4));
     if (e == cudaSuccess) e = cudaMalloc(&o, cap * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMalloc(&s.d_tiles, tile_capacity(cap) * sizeof(TileEntry));
     if (e != cudaSuccess) {
       if (p) cudaFree(p);
       if (c) cudaFree(c);
+      if (o) cudaFree(o);
       return fail(SVO_ERR_OOM, "scratch for %llu rays: %s", cap, cudaGetErrorString(e));
     }
     s.d_fix = p;
@@ -204,6 +229,7 @@ TraceItem make_item(svo_scene *s, const float *rays, uint64_t n, svo_hit *hits, 
   it.aux = s->d_aux;
   it.clusters = s->d_cl;
   it.order = s->d_order;
+  it.sph = s->d_sph;
   it.inv64 = s->d_inv64;
   it.rays = reinterpret_cast<const float4 *>(rays);
   it.hits = reinterpret_cast<uint4 *>(hits);
@@ -283,8 +309,9 @@ svo_status tile_order_table(svo_ctx *ctx, uint32_t tiles_x, uint32_t tiles_y, ui
 
 // bounds[i]: scene bound of item i (frame of origin-based ray ordering).
 // only: the scene every item traces, or nullptr (items of several scenes).
+// host_rays: the rays lie in host memory mapped into the device.
 svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays, const float4 *const *bounds,
-                     const svo_scene *only, void *stream) {
+                     const svo_scene *only, void *stream, bool host_rays = false) {
   constexpr uint32_t kReuseNeeds = SVO_TRACE_CULL | SVO_TRACE_SORT | SVO_TRACE_FP64_FIX;
   if ((L.flags & SVO_TRACE_REUSE) && (L.flags & kReuseNeeds) != kReuseNeeds)
     return fail(SVO_ERR_ARG, "SVO_TRACE_REUSE needs CULL | SORT | FP64_FIX");
@@ -345,6 +372,26 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
                                      (uint32_t)band, it.width, rows, &it.tile_order);
     if (rc != SVO_OK) return rc;
   }
+  // Image rays: cull whole tiles first (k_tile_cull).  One launch is kept for
+  // the counting build, staged top levels and wider tiles, for a scene-grid
+  // trace with items that are not images, and for rays read over the host
+  // link (the tiles that go on would be read twice: 250,000 mapped rays take
+  // 201 us in one launch, 221 in two).
+  L.tiles = nullptr;
+  L.tile_count = reinterpret_cast<unsigned int *>(slot->d_counters + 1) + 1;
+  if (!wave && !host_rays && ctx->rays_per_lane == 1 && ctx->smem_levels == 0 && !(L.flags & SVO_TRACE_STATS) &&
+      (L.flags & (SVO_TRACE_CULL | SVO_TRACE_SORT)) == (SVO_TRACE_CULL | SVO_TRACE_SORT)) {
+    unsigned long long image_tiles = 0;
+    int parts = 0;
+    for (int i = 0; i < L.n_items; ++i) {
+      parts = std::max(parts, L.items[i].n_parts);
+      if (L.items[i].tiles_x)
+        image_tiles += (i + 1 < L.n_items ? L.items[i + 1].tile_begin : L.n_tiles) - L.items[i].tile_begin;
+    }
+    const bool most = (L.flags & SVO_TRACE_GRID) ? image_tiles == L.n_tiles : 2 * image_tiles >= L.n_tiles;
+    if (most && image_tiles >= kTileCullMin && parts >= kTileCullParts && L.n_tiles <= tile_capacity(slot->cap))
+      L.tiles = slot->d_tiles;
+  }
   L.queue = nullptr;
   L.queue_count = reinterpret_cast<unsigned int *>(slot->d_counters + kQueueCountWords);
   L.queue_tile = slot->d_counters + 3;
@@ -384,7 +431,7 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
                      wave ? kQueueCountWords * sizeof(unsigned long long) + (size_t)L.n_items * sizeof(unsigned int)
                           : 3 * sizeof(unsigned long long),
                      st));
-  if (L.flags & SVO_TRACE_GRID) {
+  if ((L.flags & SVO_TRACE_GRID) && !L.tiles) {
     GridLaunch gl;
     if (grid_jobs(L.items, L.n_items, gl) > 0) CK(launch_grid(gl, st));
   }
@@ -439,6 +486,7 @@ static RefitArgs refit_args(const svo_scene *s) {
   a.aux = s->d_aux;
   a.clusters = s->d_cl;
   a.order = s->d_order;
+  a.sph = s->d_sph;
   a.n_clusters = s->NC;
   a.bound = s->d_bound;
   a.dirty = s->d_dirty;
@@ -508,6 +556,7 @@ svo_status svo_ctx_destroy(svo_ctx *ctx) {
     if (kv.second.d_fix) cudaFree(kv.second.d_fix);
     if (kv.second.d_cand) cudaFree(kv.second.d_cand);
     if (kv.second.d_off) cudaFree(kv.second.d_off);
+    if (kv.second.d_tiles) cudaFree(kv.second.d_tiles);
     if (kv.second.d_stage) cudaFree(kv.second.d_stage);
     if (kv.second.d_order) cudaFree(kv.second.d_order);
     if (kv.second.d_queue) cudaFree(kv.second.d_queue);
@@ -728,7 +777,8 @@ svo_status scene_create(svo_ctx *ctx, int32_t n_parts, const svo_handle *asset, 
   size_t off_aux = al(off_hot + P * sizeof(PartHot));
   size_t off_cl = al(off_aux + P * sizeof(PartAux));
   size_t off_order = al(off_cl + NC * sizeof(Cluster));
-  size_t off_stat = al(off_order + P * sizeof(int32_t));
+  size_t off_sph = al(off_order + P * sizeof(int32_t));
+  size_t off_stat = al(off_sph + P * sizeof(float4));
   size_t off_lo = al(off_stat + P * sizeof(PartStatic));
   size_t off_ls = al(off_lo + P * sizeof(int32_t));
   size_t off_bd = al(off_ls + (L + 1) * sizeof(int32_t));
@@ -763,6 +813,7 @@ svo_status scene_create(svo_ctx *ctx, int32_t n_parts, const svo_handle *asset, 
   s->d_aux = reinterpret_cast<PartAux *>(s->d_mem + off_aux);
   s->d_cl = reinterpret_cast<Cluster *>(s->d_mem + off_cl);
   s->d_order = reinterpret_cast<int32_t *>(s->d_mem + off_order);
+  s->d_sph = reinterpret_cast<float4 *>(s->d_mem + off_sph);
   s->d_stat = reinterpret_cast<PartStatic *>(s->d_mem + off_stat);
   s->d_level_order = reinterpret_cast<int32_t *>(s->d_mem + off_lo);
   s->d_level_start = reinterpret_cast<int32_t *>(s->d_mem + off_ls);
@@ -1013,8 +1064,8 @@ svo_status scene_read_clusters(svo_scene *s, int32_t *n_clusters, float *sphere,
   return ok();
 }
 
-svo_status trace_rays(svo_scene *s, const float *rays, uint64_t n, svo_hit *hits, uint32_t *ray_flags,
-                      uint32_t flags, svo_trace_stats *stats, void *stream) {
+static svo_status trace_one(svo_scene *s, const float *rays, uint64_t n, svo_hit *hits, uint32_t *ray_flags,
+                            uint32_t flags, svo_trace_stats *stats, void *stream, bool host_rays) {
   if (!s) return fail(SVO_ERR_ARG, "trace_rays: scene is NULL");
   if (n == 0) return ok();
   if (!rays || !hits) return fail(SVO_ERR_ARG, "trace_rays: rays/hits is NULL");
@@ -1030,7 +1081,12 @@ svo_status trace_rays(svo_scene *s, const float *rays, uint64_t n, svo_hit *hits
   L->flags = flags;
   L->stats = (flags & SVO_TRACE_STATS) ? stats : nullptr;
   const float4 *bounds[1] = {s->d_bound};
-  return run_trace(s->ctx, *L, n, bounds, s, stream);
+  return run_trace(s->ctx, *L, n, bounds, s, stream, host_rays);
+}
+
+svo_status trace_rays(svo_scene *s, const float *rays, uint64_t n, svo_hit *hits, uint32_t *ray_flags,
+                      uint32_t flags, svo_trace_stats *stats, void *stream) {
+  return trace_one(s, rays, n, hits, ray_flags, flags, stats, stream, false);
 }
 
 svo_status trace_batch(svo_ctx *ctx, const svo_batch_item *items, int32_t n_items, uint32_t flags,
@@ -1104,8 +1160,8 @@ svo_status trace_rays_host(svo_scene *s, const float *rays_host, uint64_t n, svo
     void *dev_flags = ray_flags_host ? mapped_device_pointer(ray_flags_host) : nullptr;
     if (dev_rays && dev_hits && (!ray_flags_host || dev_flags) && !(reinterpret_cast<uintptr_t>(dev_rays) & 15) &&
         !(reinterpret_cast<uintptr_t>(dev_hits) & 15))
-      return trace_rays(s, static_cast<const float *>(dev_rays), n, static_cast<svo_hit *>(dev_hits),
-                        static_cast<uint32_t *>(dev_flags), flags & ~SVO_TRACE_DEFER_FIX, nullptr, stream);
+      return trace_one(s, static_cast<const float *>(dev_rays), n, static_cast<svo_hit *>(dev_hits),
+                       static_cast<uint32_t *>(dev_flags), flags & ~SVO_TRACE_DEFER_FIX, nullptr, stream, true);
   }
   // Otherwise the rays are copied in by the copy engines, to one of two
   // staging halves that successive calls alternate between.  A call's

@@ -97,6 +97,7 @@ struct TraceItem {
   const PartAux *aux;
   const Cluster *clusters;
   const int32_t *order;
+  const float4 *sph;    // part spheres in the order of `order` (cluster members side by side)
   const double *inv64;  // FP64 world->local rows (12 per part)
   const float4 *rays;   // 2 float4 per ray
   uint4 *hits;          // svo_hit per ray
@@ -126,6 +127,20 @@ struct QueueEntry {
   int4 cp;    // the candidates' part ids
 };
 static_assert(sizeof(QueueEntry) == 64, "QueueEntry is 64 bytes");
+constexpr int kTileParts = 28;  // parts listed per image tile (TileEntry is 64 bytes)
+
+// An image tile some part sphere may be met in, written by the tile-culling
+// launch for the trace launch: the parts whose spheres reach the tile's
+// bundle of rays, or count == kTileOpen where they are not listed (more than
+// kTileParts, or rays that no cone bounds).
+struct TileEntry {
+  uint32_t tile;   // index over all items' tiles
+  uint32_t count;
+  uint16_t part[kTileParts];
+};
+static_assert(sizeof(TileEntry) == 64, "TileEntry is 64 bytes");
+constexpr uint32_t kTileOpen = 0xFFFFFFFFu;
+
 constexpr int kQueueCountWords = 4;  // per-stream counters before the per-item queue counts (64-bit words)
 
 // Warp tiles of every item, laid out one item after another: sets each
@@ -178,6 +193,8 @@ struct TraceLaunch {
   QueueEntry *queue;                  // SVO_TRACE_WAVEFRONT: entries of every item, item i from items[i].qbase
   unsigned int *queue_count;          // SVO_TRACE_WAVEFRONT: per item, entries queued; zeroed before the launch
   unsigned long long *queue_tile;     // SVO_TRACE_WAVEFRONT: tile counter of the descent launch; zeroed
+  TileEntry *tiles;                   // tile-culled image trace: the tiles to trace (nullptr: one launch over all)
+  unsigned int *tile_count;           // their number; zeroed
 };
 
 // Kernel launchers (k_trace.cu, k_refit.cu).
@@ -235,6 +252,7 @@ struct RefitArgs {
   PartAux *aux;
   Cluster *clusters;
   int32_t *order;
+  float4 *sph;                 // part spheres in the order of `order`
   int32_t n_clusters;
   float4 *bound;  // sphere enclosing every part sphere (ray-ordering frame)
   uint8_t *dirty; // set to 1 for every part whose world pose changes (cleared by each trace)

@@ -144,6 +144,8 @@ extern "C" svo_status trace_rays_noalloc(svo_scene *s, const float *rays, uint64
   L->queue = nullptr;  // no wavefront shape on this path
   L->queue_count = nullptr;
   L->queue_tile = nullptr;
+  L->tiles = nullptr;  // nor a tile queue
+  L->tile_count = nullptr;
   // clear what the kernels expect at zero: the tile counter, the list count and the pool count
   e = cudaMemsetAsync(base, 0, 3 * sizeof(unsigned long long), st);
   if (e == cudaSuccess && (flags & SVO_TRACE_GRID)) {
