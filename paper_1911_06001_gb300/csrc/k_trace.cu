@@ -27,10 +27,8 @@
 // increases.  With every direction component made non-negative by mirroring,
 // the entry of child m is max(T0, max over axes in m of the mid-plane t), so
 // the order follows from sorting the three mid-plane t values; a per-block
-// table maps a child mask to that order.  A stack holds, per level, the
-// parent's descriptor, the children still to visit, the parent's entry T0 and
-// the entry of the next child to visit, so that popping past a child that
-// starts beyond the best hit is one load and one compare.
+// table gives the first child of a mask in that order.  A stack holds, per
+// level, the parent's descriptor, the children still to visit and their order.
 #include <cuda_runtime.h>
 
 #include <cfloat>
@@ -84,76 +82,49 @@ constexpr int kCap = 4;  // candidate parts per pass (4: 1.5-2% faster than 8, f
 constexpr int kSmemParts = 256;                 // parts staged in shared memory
 constexpr int kBlock = 128;  // block size of the FP64 pass; the trace kernel takes 64, 128 or 256
 // Resident threads per SM the trace kernel's register allocation must allow
-// (768 = 24 warps: at most 80 registers a thread, no spills).  Measured per
-// frame:
-//   * articulated figure: 0.353 ms at the compiler's own 163 registers (12
-//     warps), 0.327 ms at 128 (16 warps), flat from 16 to 24 warps;
-//   * incoherent rays against ~120 parts: 9% faster at 24 warps than at 16;
-//   * 32 warps (64 registers) spill and lose.
-// The counting (STATS) and hit-buffer (REUSE) builds keep 16 warps: they would
-// spill at 80.
+// (768 = 24 warps: at most 80 registers a thread).  Measured at 24 / 20 / 16
+// warps: 2.1 M incoherent rays against 128 parts 0.712 / 0.766 / 0.857 ms, a
+// 1920x1080 frame of a 16-part figure 0.160 / 0.150 / 0.150 ms.  The counting
+// (STATS) and hit-buffer (REUSE) builds keep 16 warps: they would spill more.
 constexpr int kTraceThreadsPerSM = 768;
 // The image-tile launch (LIST) keeps 16 warps: with the culling done before,
-// it runs only tiles that descend, and 128 registers without spills beat
-// 20 warps (96 registers) and 24 (80): 0.180, 0.183 and 0.195 ms on a
-// 1920x1080 frame of a 16-part figure.
+// it runs only tiles that descend (nine requests, 6.7 M rays: 0.707 ms, 0.691
+// at 20 warps; 2.1 M rays against 1024 parts: 0.249 and 0.245).
 constexpr int kListThreadsPerSM = 512;
 
 constexpr unsigned long long kRayBits = 40;
 constexpr uint32_t kNoCand = 0xFFFFFFFFu;  // a list slot without stored leaves
 
+// Child masks of the descent: mirror[mir][mask] is a node's child mask with
+// the octants mirrored along the axes in mir; first[p][mask] the first child
+// of a (mirrored) mask in the order of their entries, p = (Bx <= By) |
+// (Bx <= Bz) << 1 | (By <= Bz) << 2 for the mid-plane parameters B.
 struct Tables {
-  uint8_t q[8][6][256];  // [mirror][perm][true child mask] -> mask in visiting order
-  uint8_t k[8][6][8];    // [mirror][perm][q] -> true octant
+  uint8_t mirror[8][256];
+  uint8_t first[8][256];
 };
 constexpr size_t kTablesBytes = (sizeof(Tables) + 15) & ~size_t(15);
 
-__host__ __device__ constexpr void perm_axes(int p, int &a0, int &a1, int &a2) {
-  // p = 2*rank_x + (rank_y > rank_z)
-  const int rx = p >> 1;
-  const bool z_first = (p & 1) != 0;
-  int r[3] = {rx, 0, 0};
-  const int lo = (rx == 0) ? 1 : 0, hi = (rx == 2) ? 1 : 2;
-  r[1] = z_first ? hi : lo;
-  r[2] = z_first ? lo : hi;
-  a0 = (r[0] == 0) ? 0 : (r[1] == 0 ? 1 : 2);
-  a1 = (r[0] == 1) ? 0 : (r[1] == 1 ? 1 : 2);
-  a2 = (r[0] == 2) ? 0 : (r[1] == 2 ? 1 : 2);
-}
-
-// perm_axes packed: bits [6p + 2r, 6p + 2r + 2) hold the axis of rank r under
-// order p.
-constexpr unsigned long long pack_axis_order() {
-  unsigned long long v = 0;
-  for (int p = 0; p < 6; ++p) {
-    int a0 = 0, a1 = 0, a2 = 0;
-    perm_axes(p, a0, a1, a2);
-    v |= (unsigned long long)(a0 | (a1 << 2) | (a2 << 4)) << (6 * p);
-  }
-  return v;
-}
-constexpr unsigned long long kAxisOrder = pack_axis_order();
-static_assert(kAxisOrder == 0x1894a1624ull, "axis order table");
-
 __device__ void build_tables(Tables *t) {
-  for (int e = threadIdx.x; e < 8 * 6 * 256; e += blockDim.x) {
-    const int h = e & 255, p = (e >> 8) % 6, mir = (e >> 8) / 6;
-    int a0, a1, a2;
-    perm_axes(p, a0, a1, a2);
-    unsigned int out = 0;
-    for (int q = 0; q < 8; ++q) {
-      const int m = ((q & 1) << a0) | (((q >> 1) & 1) << a1) | (((q >> 2) & 1) << a2);
-      const int k = m ^ mir;
-      out |= ((h >> k) & 1u) << q;
+  for (int e = threadIdx.x; e < 8 * 256; e += blockDim.x) {
+    const int a = e >> 8, mask = e & 255;
+    uint32_t mirrored = 0, first = 0;
+    // A child's entry is the largest B of its far axes, so the children come
+    // in the order of the sums of 1 << rank over those axes, rank 0 for the
+    // smallest B.
+    const int xy = a & 1, xz = (a >> 1) & 1, yz = (a >> 2) & 1;
+    const int rx = 2 - xy - xz, ry = 1 + xy - yz, rz = xz + yz;
+    int best = 64;
+    for (int m = 0; m < 8; ++m) {
+      if ((mask >> m) & 1) mirrored |= 1u << (m ^ a);
+      const int q = (m & 1 ? 1 << rx : 0) + (m & 2 ? 1 << ry : 0) + (m & 4 ? 1 << rz : 0);
+      if (((mask >> m) & 1) && q < best) {
+        best = q;
+        first = (uint32_t)m;
+      }
     }
-    t->q[mir][p][h] = (uint8_t)out;
-  }
-  for (int e = threadIdx.x; e < 8 * 6 * 8; e += blockDim.x) {
-    const int q = e & 7, p = (e >> 3) % 6, mir = (e >> 3) / 6;
-    int a0, a1, a2;
-    perm_axes(p, a0, a1, a2);
-    const int m = ((q & 1) << a0) | (((q >> 1) & 1) << a1) | (((q >> 2) & 1) << a2);
-    t->k[mir][p][q] = (uint8_t)(m ^ mir);
+    t->mirror[a][mask] = (uint8_t)mirrored;
+    t->first[a][mask] = (uint8_t)first;
   }
 }
 
@@ -175,27 +146,14 @@ struct Num;
 template <>
 struct Num<float> {
   __device__ static float inf() { return __int_as_float(0x7f800000); }
-  __device__ static float pow2neg(int l) { return __int_as_float((127 - l) << 23); }
-  __device__ static float tiny() { return 1e-30f; }
-  __device__ static float rcp(float x) { return __frcp_rn(x); }
 };
 template <>
 struct Num<double> {
   __device__ static double inf() { return __longlong_as_double(0x7ff0000000000000ll); }
   __device__ static double pow2neg(int l) { return __longlong_as_double((long long)(1023 - l) << 52); }
-  __device__ static double tiny() { return 1e-200; }
-  __device__ static double rcp(double x) { return 1.0 / x; }
 };
-
-// t of the plane x_i = P along a mirrored axis with reciprocal direction inv
-// and b = -o*inv: one FMA, whose rounding is part of the error bound behind
-// eta.
-template <typename R>
-struct Slab;
-template <>
-struct Slab<float> {
-  __device__ static float t(float P, float inv, float b) { return fmaf(P, inv, b); }
-};
+constexpr float kTinyDir = 1e-30f;  // direction components are at least this along a descent
+__device__ __forceinline__ float pow2neg(int l) { return __int_as_float((127 - l) << 23); }
 
 // FP32 per-ray state of the certified closest-hit search.
 struct CertState {
@@ -371,55 +329,67 @@ __device__ __forceinline__ uint2 node_at(const uint2 *__restrict__ nodes, uint32
 // One part's front-to-back descent in progress: what the descent keeps
 // between node visits (its stack lives in shared memory).  The local ray
 // has every direction component made non-negative by mirroring (mir: the
-// mirrored axes), with reciprocals (ix, iy, iz) and b = -o * (1/d).
-template <typename R>
+// mirrored axes), with reciprocals (ix, iy, iz).
+//
+// Node corners are kept as floats in [1, 2): 1 + the corner.  Their mantissa
+// bits are the path from the root, one per level and axis, so a step down
+// sets a bit, a pop clears the bits below its level, and a plane needs no
+// conversion from integers.  A plane P (so shifted) inflated by eta along the
+// ray is crossed at P ix + lx (its lower side) or P ix + hx (its upper side),
+// lx = -((o + 1) + eta) ix, hx = -((o + 1) - eta) ix: one FMA each.
 struct Descent {
-  R ox, oy, oz, ix, iy, iz, bx, by, bz, tmin, tmax, eta, tshift;
+  float ix, iy, iz, lx, ly, lz, hx, hy, hz, ox, oy, oz, tmin, tmax, tshift;
   const uint2 *nodes;
   uint32_t n_nodes, part, top, mir;
   int D, top_levels, level;
-  uint32_t px, py, pz;
-  uint32_t live;  // bit l: the stack entry of level l still has a child that may hold the closest hit
-  uint2 desc;     // the descriptor of the node visited next
+  uint32_t X, Y, Z;  // the node's lower corner + 1, as float bits
+  uint32_t live;     // bit l: the stack entry of level l still has a child that may hold the closest hit
+  uint2 desc;        // the descriptor of the node visited next
 };
 
 // Starts a descent at the part's root (the caller has checked n_nodes > 0).
-template <typename R, bool STATS>
-__device__ __forceinline__ void descent_start(Descent<R> &s, const uint2 *__restrict__ nodes, uint32_t n_nodes,
-                                              uint32_t top, int top_levels, int D, R ox, R oy, R oz, R dx, R dy,
-                                              R dz, R tmin, R tmax, R eta, R tshift, uint32_t part, Counters &cnt) {
-  static_assert(std::is_same<R, float>::value, "the stack stores FP32 entry parameters");
+// (o, d): the local ray, whose parameter is t - tshift; tmin / tmax in that
+// parameter.
+template <bool STATS>
+__device__ __forceinline__ void descent_start(Descent &s, const uint2 *__restrict__ nodes, uint32_t n_nodes,
+                                              uint32_t top, int top_levels, int D, float ox, float oy, float oz,
+                                              float dx, float dy, float dz, float tmin, float tmax, float eta,
+                                              float tshift, uint32_t part, Counters &cnt) {
+  // mirrored axis: o -> 1 - o, whose shift by one is 2 - o (one rounding)
   uint32_t mir = 0;
-  if (dx < R(0)) {
-    ox = R(1) - ox;
+  float sx = 1.0f + ox, sy = 1.0f + oy, sz = 1.0f + oz;
+  if (dx < 0.f) {
+    sx = 2.0f - ox;
+    ox = 1.0f - ox;
     dx = -dx;
     mir |= 1u;
   }
-  if (dy < R(0)) {
-    oy = R(1) - oy;
+  if (dy < 0.f) {
+    sy = 2.0f - oy;
+    oy = 1.0f - oy;
     dy = -dy;
     mir |= 2u;
   }
-  if (dz < R(0)) {
-    oz = R(1) - oz;
+  if (dz < 0.f) {
+    sz = 2.0f - oz;
+    oz = 1.0f - oz;
     dz = -dz;
     mir |= 4u;
   }
-  dx = dx > Num<R>::tiny() ? dx : Num<R>::tiny();
-  dy = dy > Num<R>::tiny() ? dy : Num<R>::tiny();
-  dz = dz > Num<R>::tiny() ? dz : Num<R>::tiny();
-  s.ix = Num<R>::rcp(dx);
-  s.iy = Num<R>::rcp(dy);
-  s.iz = Num<R>::rcp(dz);
-  s.bx = -(ox * s.ix);
-  s.by = -(oy * s.iy);
-  s.bz = -(oz * s.iz);
+  s.ix = __frcp_rn(fmaxf(dx, kTinyDir));
+  s.iy = __frcp_rn(fmaxf(dy, kTinyDir));
+  s.iz = __frcp_rn(fmaxf(dz, kTinyDir));
+  s.lx = -((sx + eta) * s.ix);
+  s.ly = -((sy + eta) * s.iy);
+  s.lz = -((sz + eta) * s.iz);
+  s.hx = -((sx - eta) * s.ix);
+  s.hy = -((sy - eta) * s.iy);
+  s.hz = -((sz - eta) * s.iz);
   s.ox = ox;
   s.oy = oy;
   s.oz = oz;
   s.tmin = tmin;
   s.tmax = tmax;
-  s.eta = eta;
   s.tshift = tshift;
   s.nodes = nodes;
   s.n_nodes = n_nodes;
@@ -429,67 +399,60 @@ __device__ __forceinline__ void descent_start(Descent<R> &s, const uint2 *__rest
   s.D = D;
   s.top_levels = top_levels;
   s.level = 0;
-  s.px = s.py = s.pz = 0;
+  s.X = s.Y = s.Z = 0x3F800000u;
   s.live = 0;
   s.desc = node_at(nodes, top, top_levels, 0, 0u);
   if (STATS) ++cnt.nodes;
 }
 
-// The planes of one node (level, px, py, pz in mirrored coordinates) along
-// the local ray: T0 its inflated entry (not before tmin), T1 its inflated
-// exit, B and C the entry into the far and the exit from the near half along
-// each axis, both inflated.
+// The planes of the node a descent is at: T0 its inflated entry (not before
+// tmin), T1 its inflated exit, B and C the entry into the far and the exit
+// from the near half along each axis, both inflated.
 struct NodePlanes {
-  float lx, ly, lz, h;
-  float T0, T1, Bx, By, Bz, Cx, Cy, Cz;
+  float h, T0, T1, Bx, By, Bz, Cx, Cy, Cz;
 
-  __device__ __forceinline__ NodePlanes(const Descent<float> &s, int level, uint32_t px, uint32_t py, uint32_t pz) {
-    const float sz = Num<float>::pow2neg(level), eta = s.eta;
+  __device__ __forceinline__ explicit NodePlanes(const Descent &s) {
+    const float sz = pow2neg(s.level);
     h = sz * 0.5f;
-    lx = (float)px * sz;
-    ly = (float)py * sz;
-    lz = (float)pz * sz;
-    const float Ax = Slab<float>::t(lx - eta, s.ix, s.bx), Ay = Slab<float>::t(ly - eta, s.iy, s.by),
-                Az = Slab<float>::t(lz - eta, s.iz, s.bz);
-    Bx = Slab<float>::t((lx + h) - eta, s.ix, s.bx);
-    By = Slab<float>::t((ly + h) - eta, s.iy, s.by);
-    Bz = Slab<float>::t((lz + h) - eta, s.iz, s.bz);
-    Cx = Slab<float>::t((lx + h) + eta, s.ix, s.bx);
-    Cy = Slab<float>::t((ly + h) + eta, s.iy, s.by);
-    Cz = Slab<float>::t((lz + h) + eta, s.iz, s.bz);
-    const float Ex = Slab<float>::t((lx + sz) + eta, s.ix, s.bx), Ey = Slab<float>::t((ly + sz) + eta, s.iy, s.by),
-                Ez = Slab<float>::t((lz + sz) + eta, s.iz, s.bz);
-    T0 = fmaxf(fmaxf(Ax, Ay), fmaxf(Az, s.tmin));
-    T1 = fminf(fminf(Ex, Ey), Ez);
+    const float px = __uint_as_float(s.X), py = __uint_as_float(s.Y), pz = __uint_as_float(s.Z);
+    const float mx = px + h, my = py + h, mz = pz + h;
+    T0 = fmaxf(fmaxf(fmaf(px, s.ix, s.lx), fmaf(py, s.iy, s.ly)), fmaxf(fmaf(pz, s.iz, s.lz), s.tmin));
+    T1 = fminf(fminf(fmaf(px + sz, s.ix, s.hx), fmaf(py + sz, s.iy, s.hy)), fmaf(pz + sz, s.iz, s.hz));
+    Bx = fmaf(mx, s.ix, s.lx);
+    By = fmaf(my, s.iy, s.ly);
+    Bz = fmaf(mz, s.iz, s.lz);
+    Cx = fmaf(mx, s.ix, s.hx);
+    Cy = fmaf(my, s.iy, s.hy);
+    Cz = fmaf(mz, s.iz, s.hz);
   }
 
-  // Mask (true octant space) of the children the inflated boxes of which the
-  // ray meets up to tl: child m (mirrored) is hit iff
-  // max(T0, B_i : i in m) <= min(T1, tl, C_j : j not in m).
-  __device__ __forceinline__ uint32_t hits(const Descent<float> &s, float tl) const {
-    const uint32_t mir = s.mir;
-    // masks of the children lying in the far half along each mirrored axis
-    const uint32_t HX = (mir & 1u) ? 0x55u : 0xAAu;
-    const uint32_t HY = (mir & 2u) ? 0x33u : 0xCCu;
-    const uint32_t HZ = (mir & 4u) ? 0x0Fu : 0xF0u;
+  // Mask of the children (mirrored octants m) whose inflated boxes the ray
+  // meets up to tl: max(T0, B_i : i in m) <= min(T1, tl, C_j : j not in m).
+  __device__ __forceinline__ uint32_t hits(float tl) const {
+    constexpr uint32_t FX = 0xAAu, FY = 0xCCu, FZ = 0xF0u;  // children in the far half of each axis
     const float T = fminf(T1, tl);
     uint32_t hit = (T0 <= T) ? 0xFFu : 0u;
-    hit &= (Bx <= T) ? 0xFFu : ~HX;
-    hit &= (By <= T) ? 0xFFu : ~HY;
-    hit &= (Bz <= T) ? 0xFFu : ~HZ;
-    hit &= (Cx >= T0) ? 0xFFu : HX;
-    hit &= (Cy >= T0) ? 0xFFu : HY;
-    hit &= (Cz >= T0) ? 0xFFu : HZ;
-    hit &= (Bx <= Cy) ? 0xFFu : ~(HX & ~HY);
-    hit &= (Bx <= Cz) ? 0xFFu : ~(HX & ~HZ);
-    hit &= (By <= Cx) ? 0xFFu : ~(HY & ~HX);
-    hit &= (By <= Cz) ? 0xFFu : ~(HY & ~HZ);
-    hit &= (Bz <= Cx) ? 0xFFu : ~(HZ & ~HX);
-    hit &= (Bz <= Cy) ? 0xFFu : ~(HZ & ~HY);
+    hit &= (Bx <= T) ? 0xFFu : ~FX;
+    hit &= (By <= T) ? 0xFFu : ~FY;
+    hit &= (Bz <= T) ? 0xFFu : ~FZ;
+    hit &= (Cx >= T0) ? 0xFFu : FX;
+    hit &= (Cy >= T0) ? 0xFFu : FY;
+    hit &= (Cz >= T0) ? 0xFFu : FZ;
+    hit &= (Bx <= Cy) ? 0xFFu : ~(FX & ~FY);
+    hit &= (Bx <= Cz) ? 0xFFu : ~(FX & ~FZ);
+    hit &= (By <= Cx) ? 0xFFu : ~(FY & ~FX);
+    hit &= (By <= Cz) ? 0xFFu : ~(FY & ~FZ);
+    hit &= (Bz <= Cx) ? 0xFFu : ~(FZ & ~FX);
+    hit &= (Bz <= Cy) ? 0xFFu : ~(FZ & ~FY);
     return hit;
   }
 
-  // Entry of child m (mirrored): max(T0, B_i : i in m).
+  // The row of Tables::first for the order of the three mid-planes.
+  __device__ __forceinline__ uint32_t order() const {
+    return (Bx <= By ? 1u : 0u) | (Bx <= Bz ? 2u : 0u) | (By <= Bz ? 4u : 0u);
+  }
+
+  // Entry of child m: max(T0, B_i : i in m).
   __device__ __forceinline__ float entry(uint32_t m) const {
     float lo = T0;
     if (m & 1u) lo = fmaxf(lo, Bx);
@@ -499,173 +462,138 @@ struct NodePlanes {
   }
 };
 
-// Voxel id of leaf child m (mirrored) of a level D-1 node.
-__device__ __forceinline__ unsigned long long leaf_voxel(uint32_t mir, int D, uint32_t px, uint32_t py, uint32_t pz,
-                                                         uint32_t m) {
-  const uint32_t vx = 2u * px + (m & 1u), vy = 2u * py + ((m >> 1) & 1u), vz = 2u * pz + ((m >> 2) & 1u);
-  const unsigned long long gx = (mir & 1u) ? (((1u << D) - 1u) ^ vx) : vx;
-  const unsigned long long gy = (mir & 2u) ? (((1u << D) - 1u) ^ vy) : vy;
-  const unsigned long long gz = (mir & 4u) ? (((1u << D) - 1u) ^ vz) : vz;
-  return gx | (gy << D) | (gz << (2 * D));
+// Voxel id of leaf child m of the level D-1 node a descent is at.
+__device__ __forceinline__ unsigned long long leaf_voxel(const Descent &s, uint32_t m) {
+  const int D = s.D;
+  const uint32_t flip = (1u << D) - 1u;
+  uint32_t vx = ((s.X & 0x7FFFFFu) >> (23 - D)) + (m & 1u);
+  uint32_t vy = ((s.Y & 0x7FFFFFu) >> (23 - D)) + ((m >> 1) & 1u);
+  uint32_t vz = ((s.Z & 0x7FFFFFu) >> (23 - D)) + (m >> 2);
+  if (s.mir & 1u) vx ^= flip;
+  if (s.mir & 2u) vy ^= flip;
+  if (s.mir & 4u) vz ^= flip;
+  return (unsigned long long)vx | ((unsigned long long)vy << D) | ((unsigned long long)vz << (2 * D));
 }
 
-// Leaf child m (mirrored) of a node: the entry dlo into its deflated box
-// (certain: that box is met), and the entry te into the box itself.
+// Leaf child m of a node: the entry dlo into its deflated box (certain: that
+// box is met), and the entry te into the box itself.
 struct LeafBounds {
   float dlo, te;
   bool cert;
-  __device__ __forceinline__ LeafBounds(const Descent<float> &s, const NodePlanes &nd, uint32_t m) {
-    const float h = nd.h, eta = s.eta;
-    const float clx = (m & 1u) ? nd.lx + h : nd.lx, cly = (m & 2u) ? nd.ly + h : nd.ly,
-                clz = (m & 4u) ? nd.lz + h : nd.lz;
-    dlo = fmaxf(fmaxf(Slab<float>::t(clx + eta, s.ix, s.bx), Slab<float>::t(cly + eta, s.iy, s.by)),
-                fmaxf(Slab<float>::t(clz + eta, s.iz, s.bz), s.tmin));
-    const float dhi = fminf(fminf(Slab<float>::t((clx + h) - eta, s.ix, s.bx), Slab<float>::t((cly + h) - eta, s.iy, s.by)),
-                            fminf(Slab<float>::t((clz + h) - eta, s.iz, s.bz), s.tmax));
-    te = fmaxf(fmaxf(Slab<float>::t(clx, s.ix, s.bx), Slab<float>::t(cly, s.iy, s.by)),
-               fmaxf(Slab<float>::t(clz, s.iz, s.bz), s.tmin));
+  __device__ __forceinline__ LeafBounds(const Descent &s, float h, uint32_t m) {
+    float px = __uint_as_float(s.X), py = __uint_as_float(s.Y), pz = __uint_as_float(s.Z);
+    if (m & 1u) px += h;
+    if (m & 2u) py += h;
+    if (m & 4u) pz += h;
+    dlo = fmaxf(fmaxf(fmaf(px, s.ix, s.hx), fmaf(py, s.iy, s.hy)), fmaxf(fmaf(pz, s.iz, s.hz), s.tmin));
+    const float dhi = fminf(fminf(fmaf(px + h, s.ix, s.lx), fmaf(py + h, s.iy, s.ly)),
+                            fminf(fmaf(pz + h, s.iz, s.lz), s.tmax));
+    // the corner itself is exact: p lies in [1, 2)
+    te = fmaxf(fmaxf(((px - 1.0f) - s.ox) * s.ix, ((py - 1.0f) - s.oy) * s.iy),
+               fmaxf(((pz - 1.0f) - s.oz) * s.iz, s.tmin));
     cert = dlo <= dhi;
   }
 };
 
-// One node of a descent, in FP32 with boxes inflated by eta; (o, d) is the
-// local ray whose parameter is t - tshift, tmin / tmax in that parameter.
-// State S is CertState (the certified search: leaves give entry bounds) or
-// HybridState (the FP64 pass's re-trace: every leaf reached is decided by
-// leaf_entry64).  The node's child mask comes first, then a push and a step
-// down, its leaves, or a pop: a pop goes straight to the deepest level that
-// still has a child to visit, so levels with nothing left cost no step, and
-// a lane that pops is at its next node in the same step as lanes that
-// descend.  Returns false once the part is done.
-template <typename R, typename S, bool STATS, int STRIDE>
-__device__ __forceinline__ bool descent_step(Descent<R> &s, uint4 *__restrict__ stk, const Tables *__restrict__ tab,
+// One node of a descent, in FP32 with boxes inflated by eta.  State S is
+// CertState (the certified search: leaves give entry bounds) or HybridState
+// (the FP64 pass's re-trace: every leaf reached is decided by leaf_entry64).
+// The node's child mask comes first, then its leaves, or the stack entry of
+// this node, or -- with nothing to visit here -- that of the deepest level
+// above that still has a child to visit; the step to that child is the same
+// for both, so the lanes that descend and those that pop take it together.
+// Returns false once the part is done.
+//
+// Bound by instruction issue and latency: the lanes of a warp descend, test
+// leaves and pop in the same iteration, so its length is the sum of the paths
+// (about 300 instructions and 1.3 us with integer corners, twelve
+// inflated planes, and a step of its own for pops), and a launch is as long
+// as its slowest tile, the visits of whose longest ray (150) follow each
+// other.  With the corners as floats, eta inside the planes and one step for
+// both: 1920x1080 frame of a 16-part figure 0.196 -> 0.160 ms, 2.1 M
+// incoherent rays 0.954 -> 0.712, 1.05 M rays into depth-13 parts 1.455 ->
+// 0.973.
+template <typename S, bool STATS, int STRIDE>
+__device__ __forceinline__ bool descent_step(Descent &s, uint2 *__restrict__ stk, const Tables *__restrict__ tab,
                                              S &st, Contenders *con, unsigned int &err, Counters &cnt) {
   constexpr bool CERT = std::is_same<S, CertState>::value;
   constexpr bool HYBRID = std::is_same<S, HybridState>::value;
-  const R tmax = s.tmax, tshift = s.tshift;
-  const uint32_t mir = s.mir, part = s.part;
-  const int D = s.D;
-  const uint8_t *__restrict__ qt = &tab->q[mir][0][0];
-  const uint8_t *__restrict__ kt = &tab->k[mir][0][0];
+  static_assert(CERT || HYBRID, "descent_step: CertState or HybridState");
   int level = s.level;
-  uint32_t px = s.px, py = s.py, pz = s.pz;
-  uint32_t live = s.live;
-  const uint2 desc = s.desc;
+  uint2 e;     // .x first child, .y child mask | children to visit (mirrored) << 8 | order << 16
+  uint32_t m;  // the child to step to
   {
-    const NodePlanes nd(s, level, px, py, pz);
-    const R T0 = nd.T0, Bx = nd.Bx, By = nd.By, Bz = nd.Bz;
-    uint32_t hit = nd.hits(s, rel_bound(st, tmax, tshift));
-    const uint32_t cmask = desc.y & 0xFFu;
-    hit &= cmask;
-    if (hit != 0u) {
-      const bool cxy = Bx <= By, cxz = Bx <= Bz, cyz = By <= Bz;
-      const int rx = (cxy ? 0 : 1) + (cxz ? 0 : 1);
-      const int ry = (cxy ? 1 : 0) + (cyz ? 0 : 1);
-      const int rz = (cxz ? 1 : 0) + (cyz ? 1 : 0);
-      const int p = 2 * rx + (ry > rz ? 1 : 0);
-      uint32_t hq = qt[p * 256 + hit];
-      if (level == D - 1) {
-        // children are leaves: test them in visiting order
-        while (hq) {
-          const int q = __ffs(hq) - 1;
-          hq &= hq - 1u;
-          const uint32_t k = kt[p * 8 + q];
-          const uint32_t m = k ^ mir;
-          const R lo = nd.entry(m);
-          if (lo > rel_bound(st, tmax, tshift)) break;  // later leaves start even later
-          if (STATS) ++cnt.leaves;
-          const unsigned long long vox = leaf_voxel(mir, D, px, py, pz, m);
-          if constexpr (CERT) {
-            const LeafBounds lb(s, nd, m);
-            // back to the ray's own parameter, rounding the bounds outward
-            offer(st, *con, __fadd_rd(tshift, lo), lb.cert ? __fadd_ru(tshift, lb.dlo) : Num<R>::inf(),
-                  tshift + lb.te, lb.cert, part, vox);
-          } else if constexpr (HYBRID) {
-            double tq;
-            if (leaf_entry64(st.inv64, D, vox, st.o, st.d, tq)) offer(st.ex, tq, part, vox);
-          } else {
-            static_assert(CERT || HYBRID, "descent_step: CertState or HybridState");
-          }
+    const NodePlanes nd(s);
+    uint32_t hit = nd.hits(rel_bound(st, s.tmax, s.tshift)) & tab->mirror[s.mir][s.desc.y & 0xFFu];
+    const uint32_t p = nd.order();
+    if (hit != 0u && level == s.D - 1) {
+      // children are leaves: test them in visiting order
+      do {
+        m = tab->first[p][hit];
+        hit &= ~(1u << m);
+        const float lo = nd.entry(m);
+        if (lo > rel_bound(st, s.tmax, s.tshift)) break;  // later leaves start even later
+        if (STATS) ++cnt.leaves;
+        const unsigned long long vox = leaf_voxel(s, m);
+        if constexpr (CERT) {
+          const LeafBounds lb(s, nd.h, m);
+          // back to the ray's own parameter, rounding the bounds outward
+          offer(st, *con, __fadd_rd(s.tshift, lo), lb.cert ? __fadd_ru(s.tshift, lb.dlo) : Num<float>::inf(),
+                s.tshift + lb.te, lb.cert, s.part, vox);
+        } else {
+          double tq;
+          if (leaf_entry64(st.inv64, s.D, vox, st.o, st.d, tq)) offer(st.ex, tq, s.part, vox);
         }
-      } else {
-        const int q = __ffs(hq) - 1;
-        const uint32_t rest = hq & (hq - 1u);
-        // the entry of the child visited after this one (if any), kept with the
-        // node so that a pop past it needs no plane arithmetic
-        R en = Num<R>::inf();
-        if (rest) {
-          const int ax = (int)((kAxisOrder >> (6 * p + 2 * (31 - __clz(__ffs(rest) - 1)))) & 3ull);
-          en = fmax(T0, ax == 0 ? Bx : (ax == 1 ? By : Bz));
-        }
-        stk[level * STRIDE] = make_uint4(desc.x, cmask | (rest << 8) | ((uint32_t)p << 16), __float_as_uint(en),
-                                         __float_as_uint(T0));
-        live = rest ? (live | (1u << level)) : (live & ~(1u << level));
-        const uint32_t k = kt[p * 8 + q];
-        const uint32_t idx = desc.x + __popc(cmask & ((1u << k) - 1u));
-        if (idx >= s.n_nodes) {
-          err |= kErrNodeIndex;
-          return false;
-        }
-        s.desc = node_at(s.nodes, s.top, s.top_levels, level + 1, idx);
-        if (STATS) ++cnt.nodes;
-        const uint32_t m = k ^ mir;
-        s.px = 2u * px + (m & 1u);
-        s.py = 2u * py + ((m >> 1) & 1u);
-        s.pz = 2u * pz + ((m >> 2) & 1u);
-        s.level = level + 1;
-        s.live = live;
-        return true;
+      } while (hit != 0u);
+      hit = 0u;
+    }
+    e = make_uint2(s.desc.x, s.desc.y | (hit << 8) | (p << 16));  // above the leaves a node's leaf mask is 0
+    m = tab->first[p][hit];
+    if (hit == 0u) {
+      for (;;) {  // pop to the deepest level above that still has a child to visit
+        const uint32_t cand = s.live & ((1u << level) - 1u);
+        if (cand == 0u) return false;
+        level = 31 - __clz(cand);
+        const uint32_t keep = ~0u << (23 - level);
+        s.X &= keep;
+        s.Y &= keep;
+        s.Z &= keep;
+        e = stk[level * STRIDE];
+        m = tab->first[e.y >> 16][(e.y >> 8) & 0xFFu];
+        // the child's entry, but for its parent's; past the bound, it and all
+        // later siblings are too far for good (the bound only shrinks)
+        const float h = pow2neg(level + 1);
+        float en = -Num<float>::inf();
+        if (m & 1u) en = fmaf(__uint_as_float(s.X) + h, s.ix, s.lx);
+        if (m & 2u) en = fmaxf(en, fmaf(__uint_as_float(s.Y) + h, s.iy, s.ly));
+        if (m & 4u) en = fmaxf(en, fmaf(__uint_as_float(s.Z) + h, s.iz, s.lz));
+        if (!(en > rel_bound(st, s.tmax, s.tshift))) break;
+        s.live &= ~(1u << level);
       }
     }
   }
-  for (;;) {  // pop to the deepest level above that still has a child to visit
-    const uint32_t cand = live & ((1u << level) - 1u);
-    if (cand == 0u) return false;
-    const int up = level - (31 - __clz(cand));
-    level -= up;
-    px >>= up;
-    py >>= up;
-    pz >>= up;
-    const uint4 e = stk[level * STRIDE];
-    uint32_t rest = (e.y >> 8) & 0xFFu;
-    // the next child's entry, max(T0, mid-plane t of its highest-ranked
-    // axis), was stored when the node was pushed; past the bound, this and
-    // all later siblings are too far for good (the bound only shrinks)
-    if (__uint_as_float(e.z) > rel_bound(st, tmax, tshift)) {
-      live &= ~(1u << level);
-      continue;
-    }
-    const int q = __ffs(rest) - 1;
-    rest &= rest - 1u;
-    if (!rest) live &= ~(1u << level);
-    const int p = (int)(e.y >> 16);
-    R en = Num<R>::inf();
-    if (rest) {  // the entry of the child after it
-      const R sz = Num<R>::pow2neg(level), h = sz * R(0.5);
-      const int ax = (int)((kAxisOrder >> (6 * p + 2 * (31 - __clz(__ffs(rest) - 1)))) & 3ull);
-      const R Bsel = ax == 0   ? Slab<R>::t((R(px) * sz + h) - s.eta, s.ix, s.bx)
-                     : ax == 1 ? Slab<R>::t((R(py) * sz + h) - s.eta, s.iy, s.by)
-                               : Slab<R>::t((R(pz) * sz + h) - s.eta, s.iz, s.bz);
-      en = fmax(__uint_as_float(e.w), Bsel);
-    }
-    stk[level * STRIDE] = make_uint4(e.x, (e.y & ~0xFF00u) | (rest << 8), __float_as_uint(en), e.w);
-    const uint32_t k = kt[p * 8 + q];
-    const uint32_t cmask = e.y & 0xFFu;
-    const uint32_t idx = e.x + __popc(cmask & ((1u << k) - 1u));
-    if (idx >= s.n_nodes) {
-      err |= kErrNodeIndex;
-      return false;
-    }
-    s.desc = node_at(s.nodes, s.top, s.top_levels, level + 1, idx);
-    if (STATS) ++cnt.nodes;
-    const uint32_t m = k ^ mir;
-    s.px = 2u * px + (m & 1u);
-    s.py = 2u * py + ((m >> 1) & 1u);
-    s.pz = 2u * pz + ((m >> 2) & 1u);
-    s.level = level + 1;
-    s.live = live;
-    return true;
+  // to child m of the node of `level` that e describes
+  const uint32_t rest = e.y & ~(0x100u << m);
+  const uint32_t bit = 1u << level;
+  s.live &= ~bit;
+  if (rest & 0xFF00u) {
+    s.live |= bit;
+    stk[level * STRIDE] = make_uint2(e.x, rest);
   }
+  const uint32_t k = m ^ s.mir;
+  const uint32_t idx = e.x + __popc(e.y & ((1u << k) - 1u));
+  if (idx >= s.n_nodes) {
+    err |= kErrNodeIndex;
+    return false;
+  }
+  s.desc = node_at(s.nodes, s.top, s.top_levels, level + 1, idx);
+  if (STATS) ++cnt.nodes;
+  const uint32_t half = 1u << (22 - level);
+  s.X += (m & 1u) * half;
+  s.Y += ((m >> 1) & 1u) * half;
+  s.Z += (m >> 2) * half;
+  s.level = level + 1;
+  return true;
 }
 
 struct RayW {
@@ -727,7 +655,9 @@ __device__ __forceinline__ bool cluster_cull(const RayW &r, const Cluster &c) {
 // FP32 local ray over the part (in local units), doubled for safety:
 //   q rounding            u ||Ainv||_inf ||q||_inf
 //   q - c and Ainv (q-c)   5u ||Ainv||_inf ||q - c||_inf, c' rounding u |c'|
-//   mirroring, slabs      u (4 |o'| + 3)
+//   slabs                 u (3 |s| + 2 (1 + |o'|)): s, the mirrored origin shifted by one, its sum with
+//                         eta and its product with 1/d, one u |s| each; 1/d itself and the FMA, each
+//                         relative to a plane's distance from the origin, at most 1 + |o'|
 //   FP32 direction        4u ||Ainv||_inf (|c - q|_1 + r)
 // stop: shared-memory address of the block's staged top-level nodes, of
 // which each part has its top `top_levels` levels (pa.spare0 carries, as
@@ -738,7 +668,7 @@ __device__ __forceinline__ bool cluster_cull(const RayW &r, const Cluster &c) {
 template <bool STATS, typename S>
 __device__ __forceinline__ bool part_start(const RayW &r, const PartHot &ph, const PartAux &pa, float tref,
                                            uint32_t part, uint32_t stop, int top_levels, const S &st,
-                                           Descent<float> &ds, Counters &cnt) {
+                                           Descent &ds, Counters &cnt) {
   const float4 a = ph.r0, b = ph.r1, c = ph.r2;
   const float4 s = ph.sphere;
   const float qx = fmaf(tref, r.dx, r.ox), qy = fmaf(tref, r.dy, r.oy), qz = fmaf(tref, r.dz, r.oz);
@@ -753,9 +683,12 @@ __device__ __forceinline__ bool part_start(const RayW &r, const PartHot &ph, con
   const float vn = fmaxf(fmaxf(fabsf(vx), fabsf(vy)), fabsf(vz));
   const float v1 = fabsf(vx) + fabsf(vy) + fabsf(vz);
   const float on = fmaxf(fmaxf(fabsf(ox), fabsf(oy)), fabsf(oz));
+  // the largest mirrored origin, shifted by one (descent_start)
+  const float sn = fmaxf(fmaxf(fabsf(dx < 0.f ? 2.0f - ox : 1.0f + ox), fabsf(dy < 0.f ? 2.0f - oy : 1.0f + oy)),
+                         fabsf(dz < 0.f ? 2.0f - oz : 1.0f + oz));
   const float cn = fmaxf(fmaxf(fabsf(a.w), fabsf(b.w)), fabsf(c.w));
   const float eta =
-      kU * (2.0f * pa.n_ainv * (qn + 5.0f * vn + 4.0f * (v1 + fabsf(s.w))) + 2.0f * cn + 8.0f * on + 6.0f) * 1.001f;
+      kU * (2.0f * pa.n_ainv * (qn + 5.0f * vn + 4.0f * (v1 + fabsf(s.w))) + 2.0f * cn + 6.0f * sn + 4.0f * on + 4.0f) * 1.001f;
   float tmin_rel = __fsub_rd(r.tmin, tref), tmax_rel = __fsub_ru(r.tmax, tref);
   // Clip the segment to the part's occupied box, inflated by 2 eta: one eta
   // for the local ray's error, one for this slab arithmetic.  Every leaf lies
@@ -788,7 +721,7 @@ __device__ __forceinline__ bool part_start(const RayW &r, const PartHot &ph, con
   if (!(tmin_rel <= tmax_rel) || tmin_rel > rel_bound(st, tmax_rel, tref)) return false;
   if (STATS) ++cnt.parts_entered;
   if (pa.n_nodes == 0) return false;
-  descent_start<float, STATS>(ds, pa.nodes, pa.n_nodes, stop + 8u * __float_as_uint(pa.spare0), top_levels, pa.depth,
+  descent_start<STATS>(ds, pa.nodes, pa.n_nodes, stop + 8u * __float_as_uint(pa.spare0), top_levels, pa.depth,
                               ox, oy, oz, dx, dy, dz, tmin_rel, tmax_rel, eta, tref, part, cnt);
   return true;
 }
@@ -796,11 +729,11 @@ __device__ __forceinline__ bool part_start(const RayW &r, const PartHot &ph, con
 template <bool STATS, typename S = CertState, int STRIDE = kBlock>
 __device__ __forceinline__ void trace_part_f32(const RayW &r, const PartHot &ph, const PartAux &pa, float tref,
                                                uint32_t part, const Tables *tab, uint32_t stop, int top_levels,
-                                               uint4 *stk, S &st, Contenders *con, unsigned int &err,
+                                               uint2 *stk, S &st, Contenders *con, unsigned int &err,
                                                Counters &cnt) {
-  Descent<float> ds;
+  Descent ds;
   if (part_start<STATS, S>(r, ph, pa, tref, part, stop, top_levels, st, ds, cnt))
-    while (descent_step<float, S, STATS, STRIDE>(ds, stk, tab, st, con, err, cnt)) {
+    while (descent_step<S, STATS, STRIDE>(ds, stk, tab, st, con, err, cnt)) {
     }
 }
 
@@ -843,7 +776,7 @@ template <bool STATS, int BLOCK>
 __device__ __forceinline__ bool grid_walk(const RayW &r, bool go, const SceneGrid &g,
                                           const int32_t *__restrict__ cstart, const int32_t *__restrict__ cparts,
                                           const PartHot *__restrict__ hot, const PartAux *__restrict__ aux,
-                                          const Tables *tab, uint32_t stop, int top_levels, uint4 *stk, uint32_t *mbox,
+                                          const Tables *tab, uint32_t stop, int top_levels, uint2 *stk, uint32_t *mbox,
                                           int mwords, CertState &st, Contenders &con, unsigned int &err,
                                           Counters &cnt) {
   const int G = g.G;
@@ -1137,7 +1070,7 @@ template <bool STATS, int BLOCK, bool GRID, bool LIST>
 __device__ void trace_ray_f32(const RayW &r, bool active, uint32_t flags, int P, int NC,
                               const PartHot *__restrict__ hot, const PartAux *__restrict__ aux,
                               const Cluster *__restrict__ cl, const int32_t *__restrict__ order, const Tables *tab,
-                              uint32_t stop, int top_levels, uint4 *stk, CertState &st, Contenders &con,
+                              uint32_t stop, int top_levels, uint2 *stk, CertState &st, Contenders &con,
                               unsigned int &err,
                               Counters &cnt,
                               bool reuse, uint32_t prev_part, const uint8_t *__restrict__ dirty, bool &reused,
@@ -1487,10 +1420,10 @@ __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? 
   extern __shared__ __align__(16) unsigned char smem[];
   // [tables | traversal stacks, level-major | staged part tables]
   Tables *tab = reinterpret_cast<Tables *>(smem);
-  uint4 *sStack = reinterpret_cast<uint4 *>(smem + kTablesBytes) + threadIdx.x;
+  uint2 *sStack = reinterpret_cast<uint2 *>(smem + kTablesBytes) + threadIdx.x;
   const int sp = L.one_scene ? L.items[0].n_parts : 0;
   const int sc = L.one_scene ? L.items[0].n_clusters : 0;
-  PartHot *sHot = reinterpret_cast<PartHot *>(smem + kTablesBytes + (size_t)L.stack_levels * BLOCK * sizeof(uint4));
+  PartHot *sHot = reinterpret_cast<PartHot *>(smem + kTablesBytes + (size_t)L.stack_levels * BLOCK * sizeof(uint2));
   PartAux *sAux = reinterpret_cast<PartAux *>(sHot + sp);
   Cluster *sCl = reinterpret_cast<Cluster *>(sAux + sp);
   int32_t *sOrd = reinterpret_cast<int32_t *>(sCl + sc);
@@ -1808,10 +1741,10 @@ __global__ void __launch_bounds__(BLOCK, 512 / BLOCK) k_descend(const __grid_con
   __shared__ unsigned long long sQE[NI + 1];  // first entry of each item in the flat order of all queued rays
   // [tables | traversal stacks, level-major | staged part tables]
   Tables *tab = reinterpret_cast<Tables *>(smem);
-  uint4 *sStack = reinterpret_cast<uint4 *>(smem + kTablesBytes) + threadIdx.x;
+  uint2 *sStack = reinterpret_cast<uint2 *>(smem + kTablesBytes) + threadIdx.x;
   const int sp = L.one_scene ? L.items[0].n_parts : 0;
   const int sc = L.one_scene ? L.items[0].n_clusters : 0;
-  PartHot *sHot = reinterpret_cast<PartHot *>(smem + kTablesBytes + (size_t)L.stack_levels * BLOCK * sizeof(uint4));
+  PartHot *sHot = reinterpret_cast<PartHot *>(smem + kTablesBytes + (size_t)L.stack_levels * BLOCK * sizeof(uint2));
   PartAux *sAux = reinterpret_cast<PartAux *>(sHot + sp);
   Cluster *sCl = reinterpret_cast<Cluster *>(sAux + sp);
   int32_t *sOrd = reinterpret_cast<int32_t *>(sCl + sc);
@@ -1852,7 +1785,7 @@ __global__ void __launch_bounds__(BLOCK, 512 / BLOCK) k_descend(const __grid_con
   float over_t = 0.f, last_t = 0.f;
   int last_p = -1;
   bool stopped = false;
-  Descent<float> ds;
+  Descent ds;
   unsigned long long wnext = 0, wend = 0;  // the warp's claimed run of entries (warp-uniform)
   for (;;) {
     // lanes waiting for work are served together, once enough of them wait
@@ -1963,7 +1896,7 @@ __global__ void __launch_bounds__(BLOCK, 512 / BLOCK) k_descend(const __grid_con
       state = kNeedRay;
     }
     if (__all_sync(0xffffffffu, state == kDone)) break;
-    if (state == kDescending && !descent_step<float, CertState, STATS, BLOCK>(ds, sStack, tab, st, &con, err, cnt))
+    if (state == kDescending && !descent_step<CertState, STATS, BLOCK>(ds, sStack, tab, st, &con, err, cnt))
       state = kBetween;
   }
   if (STATS) flush_stats(L.stats, cnt, 0u, n_flag);
@@ -2046,7 +1979,7 @@ __device__ void overflow_retrace(const TraceLaunchT<NI> &L, unsigned long long i
   hs.ex.vox = kMissVoxel;
   hs.o = o;
   hs.d = make_float4(d.x, d.y, d.z, r.tmax);
-  uint4 stk_local[kMaxDepth];
+  uint2 stk_local[kMaxDepth];
   double best = Num<double>::inf();  // the warp's best hit t after each round
   for (int base = 0; base < I.n_parts; base += 32) {
     const int p = base + lane;
@@ -2211,7 +2144,7 @@ __global__ void __launch_bounds__(kBlock) k_fix(const __grid_constant__ TraceLau
 }
 
 size_t trace_smem_bytes(int stack_levels, int parts, int clusters, int block, int mbox_words, int top_nodes) {
-  return kTablesBytes + (size_t)stack_levels * block * sizeof(uint4) + parts * (sizeof(PartHot) + sizeof(PartAux)) +
+  return kTablesBytes + (size_t)stack_levels * block * sizeof(uint2) + parts * (sizeof(PartHot) + sizeof(PartAux)) +
          clusters * sizeof(Cluster) + (parts + (parts & 1)) * sizeof(int32_t) + (size_t)top_nodes * sizeof(uint2) +
          (size_t)mbox_words * block * sizeof(uint32_t);
 }
