@@ -137,7 +137,8 @@ __global__ void __launch_bounds__(kGridThreads) k_build_grid(const __grid_consta
     }
   }
   __syncthreads();
-  const bool fits = any && gcnt[NC3] <= grid->cap;
+  const int gcnt_total = gcnt[NC3];
+  const bool fits = any && gcnt_total <= grid->cap;
   for (int i = tid; i < P && fits; i += kGridThreads) {
     const float4 s = job.hot[i].sphere;
     if (s.w < 0.f) continue;
@@ -170,6 +171,7 @@ __global__ void __launch_bounds__(kGridThreads) k_build_grid(const __grid_consta
       grid->inv_cs[k] = inv[k];
     }
     grid->valid = fits ? 1 : 0;
+    grid->sparse = gcnt_total <= kGridSparse * NC3 ? 1 : 0;
     grid->stale = 0;
   }
 }

@@ -273,6 +273,7 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
       const float4 sph = make_float4(cfx, cfy, cfz, (ok && ps.n_nodes > 0) ? rad : -1.0f);
       reinterpret_cast<float4 *>(&a.hot[p])[3] = sph;
       sm.sph[p] = sph;
+      a.sphere[p] = sph;
       PartAux x;
       x.nodes = ps.nodes;
       x.n_nodes = ps.n_nodes;

@@ -85,10 +85,13 @@ struct SceneGrid {
   int32_t valid;    // 0: the lists overflowed or the grid is too far from the origin: trace by clusters
   int32_t cap;      // capacity of cell_parts
   int32_t stale;    // 1: a refit changed the spheres since the last build
+  int32_t sparse;   // 1: at most kGridSparse entries per cell on average
   int32_t *cell_start;  // G^3 + 1
   int32_t *cell_parts;
 };
-constexpr int kGridMinParts = 64;  // scenes from this size on get a grid
+constexpr int kGridMinParts = 16;      // scenes from this size on get a grid
+constexpr int kGridWalkMinParts = 64;  // and from this one on SVO_TRACE_GRID walks it
+constexpr int kGridSparse = 2;
 constexpr int kGridMaxG = 16;
 
 // One item of a trace launch (by value in the kernel parameters).
@@ -98,6 +101,7 @@ struct TraceItem {
   const Cluster *clusters;
   const int32_t *order;
   const float4 *sph;    // part spheres in the order of `order` (cluster members side by side)
+  const float4 *sphere; // part spheres by part
   const double *inv64;  // FP64 world->local rows (12 per part)
   const float4 *rays;   // 2 float4 per ray
   uint4 *hits;          // svo_hit per ray
@@ -253,6 +257,7 @@ struct RefitArgs {
   Cluster *clusters;
   int32_t *order;
   float4 *sph;                 // part spheres in the order of `order`
+  float4 *sphere;              // part spheres by part
   int32_t n_clusters;
   float4 *bound;  // sphere enclosing every part sphere (ray-ordering frame)
   uint8_t *dirty; // set to 1 for every part whose world pose changes (cleared by each trace)

@@ -121,6 +121,7 @@ extern "C" svo_status trace_rays_noalloc(svo_scene *s, const float *rays, uint64
   TraceLaunch *L = &launch;
   L->items[0] = scene_item(s, rays, n, hits, ray_flags);
   if (flags & SVO_TRACE_IMAGE_TILES) L->items[0].width = flags >> 16;
+  if (L->items[0].n_parts < kGridWalkMinParts) L->items[0].grid = nullptr;
   L->n_items = 1;
   L->flags = flags;
   L->stats = nullptr;
