@@ -1,4 +1,5 @@
-// k_refit.cu -- per-frame pose pipeline of a scene, one thread block.
+// k_refit.cu -- per-frame pose pipeline of a scene, one thread block or a
+// cluster of up to eight.
 //
 //  1. compose the transform tree in FP64, parents first: W_i = W_parent(i) o L_i
 //     (the paper gives one transform per SVO, Sec. III; the tree is a
@@ -26,7 +27,17 @@
 // (b) keeps FP64 for what must be exact -- compose, inverse, sphere centre
 // and its local coordinates -- and computes the radii and norms in FP32 with
 // upward-rounded error bounds, which only ever enlarge them.
+//
+// From 65 parts on a scene gets a cluster of blocks, each on an SM of its
+// own: one SM's FP64 pipes took 110 of the 153 us of a 1024-part refit.  Every
+// block composes the whole tree (roots are copies; a level barrier inside one
+// block is cheaper than one across the cluster), inverts and bounds its share
+// of the parts, and the blocks exchange spheres, order and clusters through
+// global memory between cluster barriers.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include <cfloat>
 #include <cmath>
@@ -41,6 +52,7 @@ namespace {
 
 constexpr int kRefitThreads = 256;  // 8 warps: every FP64 sub-partition of the SM gets work
 constexpr int kRefitWarps = kRefitThreads / 32;
+constexpr int kMaxRefitCluster = 8;  // blocks of a scene's cluster
 constexpr int kQuadsPerPass = kRefitThreads / 4;  // parts handled at once (4 lanes each, 3 busy)
 constexpr float kRelSlack = 9.5367431640625e-7f;   // 2^-20: covers FP32 rounding of the norms below
 
@@ -124,20 +136,36 @@ __device__ __forceinline__ float norm_up(float x, float y, float z) {
   return __fsqrt_ru(__fmaf_ru(x, x, __fmaf_ru(y, y, __fmul_ru(z, z))));
 }
 
-// The pose pipeline of one scene, run by one block.  local: where the local
+// The pose pipeline of one scene.  local: where the local
 // poses are read from; keep != nullptr: they are first copied to keep (the
 // scene's device copy, kept in step with what is composed), and with
 // read_keep the block then reads them back from there (a source in host
 // memory is read once).
+// The blocks of the launch's cluster (all of them, or one without a cluster
+// launch) share the scene's work.
 __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *local, double *keep, bool read_keep,
                                             unsigned char *refit_smem) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int P = a.n_parts;
   const int tid = threadIdx.x;
   const int lane = tid & 31;
+  const int gtid = tid + kRefitThreads * rank, gthreads = kRefitThreads * C;  // in the cluster
   const RefitSmem sm = carve(refit_smem, P, a.n_clusters, a.n_levels);
+  // all blocks' global writes before are visible to all after
+  const auto sync = [&]() {
+    if (C > 1)
+      cluster.sync();
+    else
+      __syncthreads();
+  };
   if (keep) {
-    for (int k = tid; k < P * 12; k += kRefitThreads) keep[k] = local[k];
-    if (read_keep) local = keep;  // visible to the block after the barrier below
+    for (int k = gtid; k < P * 12; k += gthreads) keep[k] = local[k];
+    if (read_keep) {
+      local = keep;  // visible to the block after the barrier below
+      if (C > 1) cluster.sync();
+    }
   }
   // tree topology to shared memory (independent loads, one round trip)
   for (int i = tid; i < P; i += kRefitThreads) {
@@ -180,7 +208,7 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
   // change flags against the poses of the previous refit (bitwise; NaN-filled
   // at creation) and the device copy of the world poses, in one pass: one
   // global round trip for the whole scene instead of one per tree level
-  for (int k = tid; k < 12 * P; k += kRefitThreads) {
+  for (int k = gtid; k < 12 * P; k += gthreads) {
     const double w = sm.world[k];
     if (__double_as_longlong(a.world[k]) != __double_as_longlong(w)) a.dirty[k / 12] = 1;
     a.world[k] = w;
@@ -190,7 +218,7 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
   //      FP32 bounds (radius, norms) through quad shuffles
   float mn[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, mx[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
   const int rr = r < 3 ? r : 2;  // lane 3 repeats row 2 (its FP64 results are not stored)
-  for (int p = q; p < P; p += kQuadsPerPass) {
+  for (int p = q + kQuadsPerPass * rank; p < P; p += kQuadsPerPass * C) {
     const double *m = sm.world + 12 * p;
     const double A0 = m[0], A1 = m[1], A2 = m[2], A3 = m[4], A4 = m[5], A5 = m[6], A6 = m[8], A7 = m[9],
                  A8 = m[10];
@@ -297,8 +325,8 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
       mx[2] = fmaxf(mx[2], cfz);
     }
   }
-  // bounding box of the sphere centres: warp shuffles, then the eight warp
-  // results through shared memory (min and max are exact in any order)
+  // bounding box of the sphere centres: warp shuffles, then the warps'
+  // results of every block (min and max are exact in any order)
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
 #pragma unroll
@@ -314,19 +342,24 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
       sm.red[(3 + k) * kRefitWarps + (tid >> 5)] = mx[k];
     }
   }
-  __syncthreads();
+  sync();
   float bb[6];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    float v = sm.red[k * kRefitWarps];
-    for (int w = 1; w < kRefitWarps; ++w) v = k < 3 ? fminf(v, sm.red[k * kRefitWarps + w]) : fmaxf(v, sm.red[k * kRefitWarps + w]);
-    bb[k] = v;
+  for (int k = 0; k < 6; ++k) bb[k] = k < 3 ? FLT_MAX : -FLT_MAX;
+  for (int b = 0; b < C; ++b) {
+    const float *red = C > 1 ? cluster.map_shared_rank(sm.red, b) : sm.red;
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      for (int w = 0; w < kRefitWarps; ++w)
+        bb[k] = k < 3 ? fminf(bb[k], red[k * kRefitWarps + w]) : fmaxf(bb[k], red[k * kRefitWarps + w]);
   }
+  if (C > 1)  // the other blocks' spheres
+    for (int i = tid; i < P; i += kRefitThreads) sm.sph[i] = a.sphere[i];
   const float bx0 = bb[0], by0 = bb[1], bz0 = bb[2];
   const float bx1 = bb[3], by1 = bb[4], bz1 = bb[5];
   const float ex = fmaxf(bx1 - bx0, 1e-30f), ey = fmaxf(by1 - by0, 1e-30f), ez = fmaxf(bz1 - bz0, 1e-30f);
   // 5. Morton keys and a rank sort (P <= kMaxParts)
-  for (int i = tid; i < P; i += kRefitThreads) {
+  for (int i = tid; i < P; i += kRefitThreads) {  // thread i holds sphere i
     const float4 s = sm.sph[i];
     const unsigned int qx = (unsigned int)fminf(fmaxf((s.x - bx0) / ex * 1023.0f, 0.0f), 1023.0f);
     const unsigned int qy = (unsigned int)fminf(fmaxf((s.y - by0) / ey * 1023.0f, 0.0f), 1023.0f);
@@ -335,68 +368,80 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
     sm.key[i] = ((unsigned long long)mc << 11) | (unsigned long long)i;
   }
   __syncthreads();
-  for (int i = tid; i < P; i += kRefitThreads) {
-    const unsigned long long k = sm.key[i];
-    int rank = 0;
-    for (int j = 0; j < P; ++j) rank += (sm.key[j] < k) ? 1 : 0;
-    sm.ord[rank] = i;
-    a.order[rank] = i;
-    a.sph[rank] = sm.sph[i];
+  // a part's rank by `per` neighbouring threads, each against its share of the keys
+  int per = 1;
+  while (per < 8 && 2 * per * P <= gthreads) per *= 2;
+  for (int w = gtid - lane; w < P * per; w += gthreads) {  // whole warps: the shuffles below need them
+    const int i = (w + lane) / per, part = (w + lane) % per;
+    const unsigned long long k = i < P ? sm.key[i] : 0ull;
+    int pos = 0;
+    for (int j = part; j < P; j += per) pos += (sm.key[j] < k) ? 1 : 0;
+    for (int o = 1; o < per; o <<= 1) pos += __shfl_xor_sync(0xffffffffu, pos, o);
+    if (i < P && part == 0) {
+      sm.ord[pos] = i;
+      a.order[pos] = i;
+      a.sph[pos] = sm.sph[i];
+    }
   }
-  __syncthreads();
-  // clusters: a sphere around the member spheres, in FP32 rounded outward
-  for (int cidx = tid; cidx < a.n_clusters; cidx += kRefitThreads) {
+  sync();
+  // clusters: a sphere around the member spheres, in FP32 rounded outward;
+  // eight lanes each, one a member
+  static_assert(kClusterSize == 8, "eight lanes a cluster");
+  for (int w = gtid - lane; w < a.n_clusters * kClusterSize; w += gthreads) {
+    const int cidx = (w + lane) >> 3, k = lane & 7;
     const int first = cidx * kClusterSize;
-    const int cnt = min(kClusterSize, P - first);
-    float lo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, hi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
-    float na = 0.f;
-    bool any = false;
-    for (int k = 0; k < cnt; ++k) {
-      const int p = sm.ord[first + k];
-      const float4 s = sm.sph[p];
-      if (s.w < 0.f) continue;
-      any = true;
-      lo[0] = fminf(lo[0], __fsub_rd(s.x, s.w));
-      lo[1] = fminf(lo[1], __fsub_rd(s.y, s.w));
-      lo[2] = fminf(lo[2], __fsub_rd(s.z, s.w));
-      hi[0] = fmaxf(hi[0], __fadd_ru(s.x, s.w));
-      hi[1] = fmaxf(hi[1], __fadd_ru(s.y, s.w));
-      hi[2] = fmaxf(hi[2], __fadd_ru(s.z, s.w));
-      na = fmaxf(na, sm.na[p]);
-    }
-    Cluster cl;
-    if (any) {
-      // any centre works: the radius is measured from it with upward rounding
-      const float Cx = 0.5f * lo[0] + 0.5f * hi[0], Cy = 0.5f * lo[1] + 0.5f * hi[1], Cz = 0.5f * lo[2] + 0.5f * hi[2];
-      float R = 0.f;
-      for (int k = 0; k < cnt; ++k) {
-        const float4 s = sm.sph[sm.ord[first + k]];
-        if (s.w < 0.f) continue;
-        R = fmaxf(R, __fadd_ru(norm_up(abs_diff_up(s.x, Cx), abs_diff_up(s.y, Cy), abs_diff_up(s.z, Cz)), s.w));
+    const int cnt = min(kClusterSize, P - first);  // not positive past the last cluster
+    const int p = k < cnt ? (C > 1 ? a.order[first + k] : sm.ord[first + k]) : -1;
+    const float4 s = p >= 0 ? sm.sph[p] : make_float4(0.f, 0.f, 0.f, -1.0f);
+    const bool in = p >= 0 && !(s.w < 0.f);
+    float lo[3], hi[3];
+    lo[0] = in ? __fsub_rd(s.x, s.w) : FLT_MAX;
+    lo[1] = in ? __fsub_rd(s.y, s.w) : FLT_MAX;
+    lo[2] = in ? __fsub_rd(s.z, s.w) : FLT_MAX;
+    hi[0] = in ? __fadd_ru(s.x, s.w) : -FLT_MAX;
+    hi[1] = in ? __fadd_ru(s.y, s.w) : -FLT_MAX;
+    hi[2] = in ? __fadd_ru(s.z, s.w) : -FLT_MAX;
+    float na = in ? (C > 1 ? a.aux[p].n_ainv : sm.na[p]) : 0.f;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+        hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
       }
-      cl.sphere = make_float4(Cx, Cy, Cz, R);
-    } else {
-      cl.sphere = make_float4(0.f, 0.f, 0.f, -1.0f);
+      na = fmaxf(na, __shfl_xor_sync(0xffffffffu, na, o));
     }
-    cl.aux = make_float4(na, 0.f, 0.f, __uint_as_float((unsigned int)first | ((unsigned int)cnt << 16)));
-    a.clusters[cidx] = cl;
-    sm.cl[cidx] = cl.sphere;
+    const bool any = hi[0] >= lo[0];
+    // any centre works: the radius is measured from it with upward rounding
+    const float Cx = 0.5f * lo[0] + 0.5f * hi[0], Cy = 0.5f * lo[1] + 0.5f * hi[1], Cz = 0.5f * lo[2] + 0.5f * hi[2];
+    float R = in ? __fadd_ru(norm_up(abs_diff_up(s.x, Cx), abs_diff_up(s.y, Cy), abs_diff_up(s.z, Cz)), s.w) : 0.f;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, o));
+    if (k == 0 && cidx < a.n_clusters) {
+      Cluster cl;
+      cl.sphere = any ? make_float4(Cx, Cy, Cz, R) : make_float4(0.f, 0.f, 0.f, -1.0f);
+      cl.aux = make_float4(na, 0.f, 0.f, __uint_as_float((unsigned int)first | ((unsigned int)cnt << 16)));
+      a.clusters[cidx] = cl;
+      sm.cl[cidx] = cl.sphere;
+    }
   }
-  __syncthreads();
-  if (tid == 0) {
+  sync();
+  if (rank == 0 && tid < 32) {
     // a sphere around all cluster spheres: the frame of origin-based ray ordering
     const float Cx = 0.5f * (bx0 + bx1), Cy = 0.5f * (by0 + by1), Cz = 0.5f * (bz0 + bz1);
     float R = 0.f;
-    for (int c = 0; c < a.n_clusters; ++c) {
-      const float4 s = sm.cl[c];
+    for (int c = lane; c < a.n_clusters; c += 32) {
+      const float4 s = C > 1 ? a.clusters[c].sphere : sm.cl[c];
       if (s.w < 0.f) continue;
       R = fmaxf(R, __fadd_ru(norm_up(abs_diff_up(s.x, Cx), abs_diff_up(s.y, Cy), abs_diff_up(s.z, Cz)), s.w));
     }
-    *a.bound = make_float4(Cx, Cy, Cz, R);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, o));
+    if (lane == 0) *a.bound = make_float4(Cx, Cy, Cz, R);
   }
   // the scene grid, if any, no longer matches the spheres: the next grid
   // trace rebuilds it first
-  if (a.grid != nullptr && tid == 0) a.grid->stale = 1;
+  if (a.grid != nullptr && gtid == 0) a.grid->stale = 1;
 }
 
 template <bool INLINE, int CAP>
@@ -407,21 +452,50 @@ __global__ void __launch_bounds__(kRefitThreads) k_refit(RefitArgs a, const __gr
   refit_scene(a, INLINE ? poses.local : a.local, INLINE ? const_cast<double *>(a.local) : nullptr, false, refit_smem);
 }
 
-// Many scenes in one launch, one block each (scene_refit_batch): block b
-// refits B.a[b], reading its local poses from B.src[b] (device or mapped
+// Many scenes in one launch, one cluster of blocks each (scene_refit_batch):
+// cluster b refits B.a[b], reading its local poses from B.src[b] (device or mapped
 // host memory) when that is set.
 struct RefitBatch {
   RefitArgs a[kRefitBatch];
   const double *src[kRefitBatch];
   int32_t n;
+  int32_t cluster;  // blocks a scene
 };
 
 __global__ void __launch_bounds__(kRefitThreads) k_refit_batch(const __grid_constant__ RefitBatch B) {
   extern __shared__ __align__(16) unsigned char refit_smem[];
-  const int b = blockIdx.x;
+  const int b = blockIdx.x / B.cluster;
   const RefitArgs &a = B.a[b];
   const double *src = B.src[b];
   refit_scene(a, src ? src : a.local, src ? const_cast<double *>(a.local) : nullptr, true, refit_smem);
+}
+
+// Blocks of a scene's cluster: a block takes 64 parts a pass, two warps on
+// each FP64 pipe.  Measured per refit, one block (of the code before) against
+// the cluster: 1024 parts 153 -> 52 us (4 blocks: 72), 128 parts 25.6 -> 19.1,
+// 64 scenes of up to 256 parts in one launch 42 -> 27 (32 parts a block: 53,
+// the launch then waits for room for its clusters).
+int refit_cluster(int n_parts) {
+  int c = 1;
+  while (c < kMaxRefitCluster && 64 * c < n_parts) c *= 2;
+  return c;
+}
+
+template <typename... Params, typename... Args>
+cudaError_t launch_clusters(void (*kern)(Params...), int n, int cluster, size_t smem, cudaStream_t stream,
+                            const Args &...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned int)(n * cluster));
+  cfg.blockDim = dim3(kRefitThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned int)cluster;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 template <bool INLINE, int CAP>
@@ -431,8 +505,7 @@ cudaError_t launch_refit_t(const RefitArgs &a, const double *host_local, size_t 
     for (int k = 0; k < a.n_parts * 12; ++k) p.local[k] = host_local[k];
   cudaError_t e = cudaFuncSetAttribute(k_refit<INLINE, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_refit<INLINE, CAP><<<1, kRefitThreads, smem, stream>>>(a, p);
-  return cudaGetLastError();
+  return launch_clusters(k_refit<INLINE, CAP>, 1, refit_cluster(a.n_parts), smem, stream, a, p);
 }
 
 }  // namespace
@@ -454,6 +527,9 @@ cudaError_t launch_refit_batch(const RefitArgs *args, const double *const *src, 
     smem = m > smem ? m : smem;
   }
   B.n = n;
+  int parts = 0;
+  for (int i = 0; i < n; ++i) parts = std::max(parts, (int)args[i].n_parts);
+  B.cluster = refit_cluster(parts);
   // the shared-memory attribute only ever grows: set it when this launch needs more (per device)
   constexpr int kMaxDevices = 64;
   static std::mutex mu;
@@ -470,8 +546,7 @@ cudaError_t launch_refit_batch(const RefitArgs *args, const double *const *src, 
       admitted[dev] = smem;
     }
   }
-  k_refit_batch<<<n, kRefitThreads, smem, stream>>>(B);
-  return cudaGetLastError();
+  return launch_clusters(k_refit_batch, n, B.cluster, smem, stream, B);
 }
 
 cudaError_t launch_refit(const RefitArgs &a, const double *host_local, cudaStream_t stream) {

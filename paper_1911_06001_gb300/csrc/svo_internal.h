@@ -269,7 +269,7 @@ struct RefitArgs {
 cudaError_t launch_refit(const RefitArgs &a, const double *host_local, cudaStream_t stream);
 // Scenes per launch of scene_refit_batch (kernel parameter space).
 constexpr int kRefitBatch = 64;
-// n <= kRefitBatch scenes in one launch, one block each; src[i]: where scene
+// n <= kRefitBatch scenes in one launch, one cluster of blocks each; src[i]: where scene
 // i's local poses are read from (device or mapped host memory), or nullptr
 // for args[i].local.
 cudaError_t launch_refit_batch(const RefitArgs *args, const double *const *src, int n, cudaStream_t stream);
