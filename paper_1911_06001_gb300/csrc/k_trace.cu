@@ -175,60 +175,52 @@ struct ExactState {
   unsigned long long vox;
 };
 
-// Closed-box entry of one leaf in FP64 (the definition the oracle follows,
-// each slab quotient taken as a product with the reciprocal of the direction
-// component): ray to the part frame with the FP64 inverse, slab test of the
-// leaf cell's box; a zero direction component keeps the slab only if the
-// origin lies in it.  Returns whether the leaf is hit and its candidate t.
-__device__ __forceinline__ bool leaf_entry64(const double *__restrict__ m, int D, unsigned long long vox, float4 o,
-                                             float4 d, double &t) {
+// A ray in a part's frame in FP64: the origin, and one reciprocal per axis
+// instead of two divisions a leaf (the result differs from the quotient by at
+// most an ulp or two); inv = 0 stands for a zero direction component.
+struct LocalRay64 {
+  double o[3], inv[3];
+};
+
+__device__ __forceinline__ LocalRay64 local_ray64(const double *__restrict__ m, float4 o, float4 d) {
   const double ox = o.x, oy = o.y, oz = o.z, dx = d.x, dy = d.y, dz = d.z;
-  const double lo3[3] = {fma(m[0], ox, fma(m[1], oy, fma(m[2], oz, m[3]))),
-                         fma(m[4], ox, fma(m[5], oy, fma(m[6], oz, m[7]))),
-                         fma(m[8], ox, fma(m[9], oy, fma(m[10], oz, m[11])))};
-  const double ld3[3] = {fma(m[0], dx, fma(m[1], dy, m[2] * dz)), fma(m[4], dx, fma(m[5], dy, m[6] * dz)),
-                         fma(m[8], dx, fma(m[9], dy, m[10] * dz))};
-  const unsigned long long mask = (1ull << D) - 1ull;
-  const double s = Num<double>::pow2neg(D);
-  double t0 = (double)o.w, t1 = (double)d.w;
+  LocalRay64 l;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const double c = (double)((vox >> (k * D)) & mask);
-    const double blo = c * s, bhi = (c + 1.0) * s;
-    if (ld3[k] == 0.0) {
-      if (lo3[k] < blo || lo3[k] > bhi) return false;
+    l.o[k] = fma(m[4 * k], ox, fma(m[4 * k + 1], oy, fma(m[4 * k + 2], oz, m[4 * k + 3])));
+    const double ld = fma(m[4 * k], dx, fma(m[4 * k + 1], dy, m[4 * k + 2] * dz));
+    l.inv[k] = ld != 0.0 ? 1.0 / ld : 0.0;
+  }
+  return l;
+}
+
+// Closed-box entry of one leaf in FP64 (the definition the oracle follows):
+// slab test of the leaf cell's box between tmin and tmax; a zero direction
+// component keeps the slab only if the origin lies in it.  Returns whether
+// the leaf is hit and its candidate t.  FP64 issues at two lanes per clock
+// and SM, so its instructions are what this costs: the near plane is picked
+// by the sign bit of the reciprocal, and the far corner is the near one plus
+// a leaf (exact).
+__device__ __forceinline__ bool leaf_entry64(const LocalRay64 &l, int D, unsigned long long vox, float tmin,
+                                             float tmax, double &t) {
+  const uint32_t mask = (1u << D) - 1u;
+  const double s = Num<double>::pow2neg(D);
+  double t0 = (double)tmin, t1 = (double)tmax;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const double blo = (double)((uint32_t)(vox >> (k * D)) & mask) * s, bhi = blo + s;
+    const long long bits = __double_as_longlong(l.inv[k]);
+    if (bits == 0) {
+      if (l.o[k] < blo || l.o[k] > bhi) return false;
       continue;
     }
-    // one reciprocal per axis instead of two divisions: FP64 issues at a few
-    // lanes per clock, so this pass is bound by its FP64 instruction count
-    // (the result differs from the quotient by at most an ulp or two)
-    const double inv = 1.0 / ld3[k];
-    double ta = (blo - lo3[k]) * inv, tb = (bhi - lo3[k]) * inv;
-    if (ta > tb) {
-      const double x = ta;
-      ta = tb;
-      tb = x;
-    }
-    t0 = fmax(t0, ta);
-    t1 = fmin(t1, tb);
+    const double ta = (blo - l.o[k]) * l.inv[k], tb = (bhi - l.o[k]) * l.inv[k];
+    const double near = bits < 0 ? tb : ta, far = bits < 0 ? ta : tb;
+    t0 = near > t0 ? near : t0;
+    t1 = far < t1 ? far : t1;
   }
   t = t0;
   return t0 <= t1;
-}
-
-// The FP64 pass for a ray whose contender list overflowed: the FP32 descent
-// with inflated boxes (as in the certified pass, so no leaf the FP64 rule could
-// hit is skipped), each leaf reached decided by leaf_entry64, and the
-// lexicographic minimum kept in FP64.  Same result as an FP64 descent, at FP32
-// speed for the interior nodes.
-struct HybridState {
-  ExactState ex;
-  const double *inv64;  // the part's FP64 world->local rows
-  float4 o, d;          // the ray as given (FP32)
-};
-
-__device__ __forceinline__ float rel_bound(const HybridState &s, float tmax_rel, float tshift) {
-  return fminf(tmax_rel, __fsub_ru(__double2float_ru(s.ex.t), tshift));
 }
 
 // Leaves that may still be the closest hit: every candidate whose entry lower
@@ -307,13 +299,6 @@ struct Counters {
   uint32_t f_winner, f_overlap, f_width, reused;
 };
 
-// Front-to-back descent of one part in its local frame, in FP32 with boxes
-// inflated by eta.  (o, d): local ray whose parameter is t - tshift;
-// tmin/tmax are in that shifted parameter.  State S is CertState (the
-// certified search: leaves give entry bounds) or HybridState (the FP64 pass's
-// re-trace: every leaf reached is decided by leaf_entry64).
-// Node descriptor idx of a part: the first ntop come from the block's
-// shared-memory copy of the part's top levels, the rest from global memory.
 // Descriptor idx, a node of level `lev`, of a part.  The node array is
 // breadth first, so the nodes of the top `top_levels` levels are its first
 // ones; those come from the block's shared-memory copy at address `top`
@@ -498,9 +483,8 @@ struct LeafBounds {
   }
 };
 
-// One node of a descent, in FP32 with boxes inflated by eta.  State S is
-// CertState (the certified search: leaves give entry bounds) or HybridState
-// (the FP64 pass's re-trace: every leaf reached is decided by leaf_entry64).
+// One node of a descent, the certified search in FP32 with boxes inflated by
+// eta: leaves give entry bounds.
 // The node's child mask comes first, then its leaves, or the stack entry of
 // this node, or -- with nothing to visit here -- that of the deepest level
 // above that still has a child to visit; the step to that child is the same
@@ -516,12 +500,9 @@ struct LeafBounds {
 // both: 1920x1080 frame of a 16-part figure 0.196 -> 0.160 ms, 2.1 M
 // incoherent rays 0.954 -> 0.712, 1.05 M rays into depth-13 parts 1.455 ->
 // 0.973.
-template <typename S, bool STATS, int STRIDE>
+template <bool STATS, int STRIDE>
 __device__ __forceinline__ bool descent_step(Descent &s, uint2 *__restrict__ stk, const Tables *__restrict__ tab,
-                                             S &st, Contenders *con, unsigned int &err, Counters &cnt) {
-  constexpr bool CERT = std::is_same<S, CertState>::value;
-  constexpr bool HYBRID = std::is_same<S, HybridState>::value;
-  static_assert(CERT || HYBRID, "descent_step: CertState or HybridState");
+                                             CertState &st, Contenders &con, unsigned int &err, Counters &cnt) {
   int level = s.level;
   uint2 e;     // .x first child, .y child mask | children to visit (mirrored) << 8 | order << 16
   uint32_t m;  // the child to step to
@@ -539,15 +520,10 @@ __device__ __forceinline__ bool descent_step(Descent &s, uint2 *__restrict__ stk
         if (lo > rel_bound(st, s.tmax, s.tshift)) break;  // later leaves start even later
         if (STATS) ++cnt.leaves;
         const unsigned long long vox = leaf_voxel(s, m);
-        if constexpr (CERT) {
-          const LeafBounds lb(s, nd.h, m);
-          // back to the ray's own parameter, rounding the bounds outward
-          offer(st, *con, __fadd_rd(s.tshift, lo), lb.cert ? __fadd_ru(s.tshift, lb.dlo) : Num<float>::inf(),
-                s.tshift + lb.te, lb.cert, s.part, vox);
-        } else {
-          double tq;
-          if (leaf_entry64(st.inv64, s.D, vox, st.o, st.d, tq)) offer(st.ex, tq, s.part, vox);
-        }
+        const LeafBounds lb(s, nd.h, m);
+        // back to the ray's own parameter, rounding the bounds outward
+        offer(st, con, __fadd_rd(s.tshift, lo), lb.cert ? __fadd_ru(s.tshift, lb.dlo) : Num<float>::inf(),
+              s.tshift + lb.te, lb.cert, s.part, vox);
       } while (hit != 0u);
       hit = 0u;
     }
@@ -738,14 +714,14 @@ __device__ __forceinline__ bool part_start(const RayW &r, const PartHot &ph, con
   return true;
 }
 
-template <bool STATS, typename S = CertState, int STRIDE = kBlock>
+template <bool STATS, int STRIDE>
 __device__ __forceinline__ void trace_part_f32(const RayW &r, const PartHot &ph, const PartAux &pa, float tref,
                                                uint32_t part, const Tables *tab, uint32_t stop, int top_levels,
-                                               uint2 *stk, S &st, Contenders *con, unsigned int &err,
+                                               uint2 *stk, CertState &st, Contenders &con, unsigned int &err,
                                                Counters &cnt) {
   Descent ds;
-  if (part_start<STATS, S>(r, ph, pa, tref, part, stop, top_levels, st, ds, cnt))
-    while (descent_step<S, STATS, STRIDE>(ds, stk, tab, st, con, err, cnt)) {
+  if (part_start<STATS, CertState>(r, ph, pa, tref, part, stop, top_levels, st, ds, cnt))
+    while (descent_step<STATS, STRIDE>(ds, stk, tab, st, con, err, cnt)) {
     }
 }
 
@@ -883,8 +859,8 @@ __device__ __forceinline__ bool grid_walk(const RayW &r, bool go, const SceneGri
 #pragma unroll 1
     for (int i = 0; i < kCap && __any_sync(0xffffffffu, ct[0] != Num<float>::inf()); ++i) {
       if (ct[0] != Num<float>::inf() && ct[0] <= prune_bound(st, r.tmax))
-        trace_part_f32<STATS, CertState, BLOCK>(r, hot[cp[0]], aux[cp[0]], ce[0], (uint32_t)cp[0], tab, stop,
-                                                top_levels, stk, st, &con, err, cnt);
+        trace_part_f32<STATS, BLOCK>(r, hot[cp[0]], aux[cp[0]], ce[0], (uint32_t)cp[0], tab, stop,
+                                                top_levels, stk, st, con, err, cnt);
 #pragma unroll
       for (int j = 0; j < kCap - 1; ++j) {
         ct[j] = ct[j + 1];
@@ -1260,8 +1236,8 @@ __device__ void trace_ray_f32(const RayW &r, bool active, uint32_t flags, int P,
             stopped = true;
             break;
           }
-          trace_part_f32<STATS, CertState, BLOCK>(r, hot[p], aux[p], eta, (uint32_t)p, tab, stop, top_levels, stk,
-                                                  st, &con, err, cnt);
+          trace_part_f32<STATS, BLOCK>(r, hot[p], aux[p], eta, (uint32_t)p, tab, stop, top_levels, stk,
+                                                  st, con, err, cnt);
           last_t = tin;
           last_p = p;
         }
@@ -1277,8 +1253,8 @@ __device__ void trace_ray_f32(const RayW &r, bool active, uint32_t flags, int P,
       const bool h = part_cull(r, hot[p], tin, tref);
       if (cull && !h) continue;
       // the plain trace descends every part, even one whose sphere is missed
-      trace_part_f32<STATS, CertState, BLOCK>(r, hot[p], aux[p], tref, (uint32_t)p, tab, stop, top_levels, stk, st,
-                                              &con, err, cnt);
+      trace_part_f32<STATS, BLOCK>(r, hot[p], aux[p], tref, (uint32_t)p, tab, stop, top_levels, stk, st,
+                                              con, err, cnt);
     }
   }
 }
@@ -2154,14 +2130,205 @@ __global__ void __launch_bounds__(BLOCK, 512 / BLOCK) k_descend(const __grid_con
       state = kNeedRay;
     }
     if (__all_sync(0xffffffffu, state == kDone)) break;
-    if (state == kDescending && !descent_step<CertState, STATS, BLOCK>(ds, sStack, tab, st, &con, err, cnt))
+    if (state == kDescending && !descent_step<STATS, BLOCK>(ds, sStack, tab, st, con, err, cnt))
       state = kBetween;
   }
   if (STATS) flush_stats(L.stats, cnt, 0u, n_flag);
   if (err) atomicOr(L.err, err);
 }
 
+// ------------------------------------------------- one ray by a whole warp
+
+// The search of one ray with its node visits spread over a warp's lanes.  The
+// ray's candidate parts are found 32 at a time and set up one per lane; their
+// roots go onto a stack of nodes in shared memory, and every round takes up to
+// 32 nodes off it, one per lane, and pushes the children the ray meets.  A
+// sink takes the leaves (leaf), prunes (bound, as rel_bound) and gathers what
+// the lanes found after every round (round).  A long chain of node visits --
+// a grazing ray's hundreds -- takes a few dozen rounds.
+//
+// The stack holds kCoopStack nodes.  While it has room for what 32 nodes can
+// push (at most 7 net each) a round takes 32; nearer to the end it takes
+// fewer, down to one at a time, for which a depth-first search needs no more
+// than 7 slots a level: the room kept back for it.
+constexpr int kCoopStack = 320;
+constexpr int kCoopParts = 16;  // candidate parts set up at a time
+constexpr int kCoopReserve = 7 * kMaxDepth + 8;
+static_assert(kCoopStack > 2 * kCoopReserve + 32, "room to work in");
+
+struct CoopWarp {
+  uint4 stack[kCoopStack];  // node | corner x, y << 16 | corner z, level << 16, part slot << 24 | entry (the part's)
+  Descent part[kCoopParts];
+};
+
+// Takes the nodes off the stack (top of them, warp-uniform) until it is empty.
+template <typename Sink>
+__device__ __forceinline__ void coop_drain(CoopWarp &w, int top, const Tables *__restrict__ tab, Sink &sink,
+                                           unsigned int &err) {
+  const int lane = threadIdx.x & 31;
+  while (top > 0) {
+    const int n = min(top, max(1, min(32, (kCoopStack - kCoopReserve - top) / 7)));
+    top -= n;
+    uint4 e = make_uint4(0u, 0u, 0u, 0u);
+    if (lane < n) e = w.stack[top + lane];
+    __syncwarp();
+    uint32_t hit = 0;  // children to push (mirrored)
+    const uint32_t slot = e.z >> 24;
+    Descent s = w.part[slot];
+    s.X = 0x3F800000u | ((e.y & 0xFFFFu) << 7);
+    s.Y = 0x3F800000u | ((e.y >> 16) << 7);
+    s.Z = 0x3F800000u | ((e.z & 0xFFFFu) << 7);
+    s.level = (int)((e.z >> 16) & 0xFFu);
+    const NodePlanes nd(s);
+    uint2 desc = make_uint2(0u, 0u);
+    if (lane < n && __uint_as_float(e.w) <= sink.bound(s)) {
+      desc = __ldg(&s.nodes[e.x]);
+      hit = nd.hits(sink.bound(s)) & tab->mirror[s.mir][desc.y & 0xFFu];
+      if (s.level == s.D - 1) {
+        for (; hit != 0u; hit &= hit - 1u) {
+          const uint32_t m = (uint32_t)__ffs(hit) - 1u;
+          if (nd.entry(m) <= sink.bound(s)) sink.leaf(s, nd, m);
+        }
+      }
+    }
+    int at = __popc(hit);
+    const int own = at;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, at, o);
+      if (lane >= o) at += v;
+    }
+    const int total = __shfl_sync(0xffffffffu, at, 31);
+    const int shift = 22 - s.level;  // the bit of a corner's float that a step down sets
+    for (int pos = top + at - own; hit != 0u; ++pos) {
+      const uint32_t m = 31u - (uint32_t)__clz(hit);  // the child nearest to the ray's start goes on top
+      hit &= ~(1u << m);
+      const uint32_t k = m ^ s.mir;
+      uint32_t idx = desc.x + __popc(desc.y & ((1u << k) - 1u));
+      float en = nd.entry(m);
+      if (idx >= s.n_nodes) {  // not followed: no bound admits this entry
+        err |= kErrNodeIndex;
+        idx = 0;
+        en = __int_as_float(0x7fffffff);
+      }
+      const uint32_t cx = ((s.X & 0x7FFFFFu) | ((m & 1u) << shift)) >> 7,
+                     cy = ((s.Y & 0x7FFFFFu) | (((m >> 1) & 1u) << shift)) >> 7,
+                     cz = ((s.Z & 0x7FFFFFu) | ((m >> 2) << shift)) >> 7;
+      w.stack[pos] = make_uint4(idx, cx | (cy << 16), cz | ((uint32_t)(s.level + 1) << 16) | (slot << 24),
+                                __float_as_uint(en));
+    }
+    top += total;
+    __syncwarp();
+    sink.round();
+  }
+}
+
+// All parts of item I.  r is the same on every lane.
+template <typename Sink>
+__device__ __forceinline__ void coop_trace(CoopWarp &w, const TraceItem &I, const RayW &r,
+                                           const Tables *__restrict__ tab, Sink &sink, unsigned int &err,
+                                           Counters &cnt) {
+  const int lane = threadIdx.x & 31;
+  int n_cand = 0;
+  for (int base = 0; base < I.n_parts; base += 32) {
+    const int p = base + lane;
+    Descent ds;
+    float tin, tref;
+    const bool in = p < I.n_parts && part_cull(r, I.hot[p], tin, tref) && !(tin > sink.best()) &&
+                    part_start<false>(r, I.hot[p], I.aux[p], tref, (uint32_t)p, 0u, 0, sink, ds, cnt);
+    for (unsigned int m = __ballot_sync(0xffffffffu, in); m != 0u;) {
+      const int c = min(__popc(m), kCoopParts - n_cand);  // as many as there are slots left
+      const int q = __popc(m & ((1u << lane) - 1u));
+      if (((m >> lane) & 1u) && q < c) {
+        w.part[n_cand + q] = ds;
+        w.stack[n_cand + q] = make_uint4(0u, 0u, (uint32_t)(n_cand + q) << 24, __float_as_uint(ds.tmin));
+      }
+      n_cand += c;
+      for (int k = 0; k < c; ++k) m &= m - 1u;  // the lowest c lanes are in
+      __syncwarp();
+      if (n_cand == kCoopParts) {
+        coop_drain(w, n_cand, tab, sink, err);
+        n_cand = 0;
+      }
+    }
+  }
+  coop_drain(w, n_cand, tab, sink, err);
+}
+
+// The exact search (the FP64 pass's re-trace): the FP32 search with inflated
+// boxes, so no leaf the FP64 rule could hit is skipped, collects the leaves it
+// reaches, and the warp decides them in FP64, 32 at a time.
+constexpr int kLeafBuf = 31 + 32 * 8;  // emptied from 32 on; a round adds at most 8 a lane
+struct LeafBuf {
+  unsigned long long vox[kLeafBuf];
+  uint32_t part[kLeafBuf];
+  unsigned int n;
+};
+
+struct ExactSink {
+  LeafBuf &buf;
+  const TraceItem &I;
+  float4 o, d;    // the ray; d.w: where the search ends
+  float closest;  // upper bound of the closest hit's t so far
+  ExactState ex;  // this lane's
+
+  __device__ __forceinline__ float best() const { return closest; }
+  __device__ __forceinline__ float bound(const Descent &s) const {
+    return fminf(s.tmax, __fsub_ru(closest, s.tshift));
+  }
+  __device__ __forceinline__ void leaf(const Descent &s, const NodePlanes &, uint32_t m) {
+    const unsigned int q = atomicAdd(&buf.n, 1u);
+    if (q < (unsigned int)kLeafBuf) {
+      buf.vox[q] = leaf_voxel(s, m);
+      buf.part[q] = s.part;
+    }
+  }
+  __device__ __forceinline__ void decide() {
+    const int lane = threadIdx.x & 31, n = (int)buf.n;
+    for (int k = lane; k < n; k += 32) {
+      const uint32_t p = buf.part[k];
+      double tq;
+      if (leaf_entry64(local_ray64(I.inv64 + 12 * p, o, d), I.aux[p].depth, buf.vox[k], o.w, d.w, tq))
+        offer(ex, tq, p, buf.vox[k]);
+    }
+    double t = ex.t;
+#pragma unroll
+    for (int q = 16; q > 0; q >>= 1) t = fmin(t, __shfl_xor_sync(0xffffffffu, t, q));
+    closest = __double2float_ru(t);
+    __syncwarp();
+    if (lane == 0) buf.n = 0;
+    __syncwarp();
+  }
+  __device__ __forceinline__ void round() {
+    if (buf.n >= 32u) decide();
+    __syncwarp();  // every lane has read the count
+  }
+};
+
+__device__ __forceinline__ float rel_bound(const ExactSink &s, float tmax_rel, float tshift) {
+  return fminf(tmax_rel, __fsub_ru(s.closest, tshift));
+}
+
 // ------------------------------------------------------------- FP64 pass
+
+// One warp's 32 list entries in the FP64 pass.
+struct FixWarp {
+  double o[3][32], inv[3][32];  // the ray in the frame of its first leaf's part
+  unsigned long long key[32], vox[32];  // one round's results
+  uint32_t part[32], first[32], off[32];
+  float tmin[32], tmax[32];
+  int depth[32], begin[32];  // begin: an entry's first place in the flat order of the other leaves
+};
+
+struct RetraceWarp {
+  CoopWarp coop;
+  LeafBuf buf;
+};
+
+union FixUnion {  // a warp does one or the other
+  FixWarp list;
+  RetraceWarp re;
+};
 
 // Lexicographic minimum of (t, part, voxel) across the warp (every lane
 // returns it).
@@ -2202,15 +2369,16 @@ __device__ __forceinline__ void group_min8(ExactState &s) {
 
 // The FP64 pass for a flagged ray without a contender list (the list
 // overflowed), called by the whole warp (i: its list index, e: its entry).
-// The warp re-traces the ray, lane q taking parts q, q + 32, ...; each lane
-// keeps the exact minimum over its parts, the warp's best hit so far prunes
-// whole parts, and a warp reduction gives the overall minimum.  The segment
-// ends at the FP32 pass's certain upper bound of the winner's t where one was
-// stored: the winner (and every leaf tied with it) starts no later, so no
-// candidate is lost and the leaves beyond it are never tested in FP64.
+// The warp re-traces the ray together (coop_trace).  The segment ends at the
+// FP32 pass's certain upper bound of the winner's t where one was stored: the
+// winner (and every leaf tied with it) starts no later, so no candidate is
+// lost and the leaves beyond it are never tested in FP64.  With the parts dealt
+// over the lanes and each lane's leaves decided as it came to them, one such
+// ray took 50 to 100 us (its node visits one after another), and the 42,600 of
+// 1.05 M rays into depth-13 parts 1.73 ms.
 template <int NI>
 __device__ void overflow_retrace(const TraceLaunchT<NI> &L, unsigned long long i, unsigned long long e,
-                                 const Tables *tab, unsigned int &err, Counters &cnt) {
+                                 const Tables *tab, FixUnion &u, unsigned int &err, Counters &cnt) {
   const int lane = threadIdx.x & 31;
   const uint32_t why = ((e >> 47) & 1ull) ? SVO_RAY_T_REFINED : SVO_RAY_UNCERTAIN;
   const int it = (int)((e >> kRayBits) & 0x7Fu);
@@ -2231,49 +2399,46 @@ __device__ void overflow_retrace(const TraceLaunchT<NI> &L, unsigned long long i
   r.inv_dd = 1.0f / (d.x * d.x + d.y * d.y + d.z * d.z);
   r.inv_len = 0.f;
   r.onorm = 0.f;
-  HybridState hs;
-  hs.ex.t = Num<double>::inf();
-  hs.ex.part = kMissPart;
-  hs.ex.vox = kMissVoxel;
-  hs.o = o;
-  hs.d = make_float4(d.x, d.y, d.z, r.tmax);
-  uint2 stk_local[kMaxDepth];
-  double best = Num<double>::inf();  // the warp's best hit t after each round
-  for (int base = 0; base < I.n_parts; base += 32) {
-    const int p = base + lane;
-    if (p < I.n_parts) {
-      float tin, tref;
-      if (part_cull(r, I.hot[p], tin, tref) && !(tin > __double2float_ru(fmin(best, hs.ex.t)))) {
-        hs.inv64 = I.inv64 + 12 * p;
-        trace_part_f32<false, HybridState, 1>(r, I.hot[p], I.aux[p], tref, (uint32_t)p, tab, 0u, 0, stk_local, hs,
-                                              nullptr, err, cnt);
-      }
-    }
-    double bb = hs.ex.t;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) bb = fmin(bb, __shfl_xor_sync(0xffffffffu, bb, off));
-    best = bb;
-  }
-  warp_min(hs.ex);
-  if (lane == 0) write_fixed(I, ray, hs.ex, why);
+  ExactSink sink = {u.re.buf, I, o, make_float4(d.x, d.y, d.z, r.tmax), Num<float>::inf(),
+                    {Num<double>::inf(), kMissPart, kMissVoxel}};
+  __syncwarp();  // the union's other member is read
+  if (lane == 0) sink.buf.n = 0;
+  __syncwarp();
+  coop_trace(u.re.coop, I, r, tab, sink, err, cnt);
+  sink.decide();
+  warp_min(sink.ex);
+  if (lane == 0) write_fixed(I, ray, sink.ex, why);
+}
+
+// A candidate's t as an unsigned integer of the same order (-0 as 0), so that
+// comparing candidates takes no FP64 instruction; kNoHitKey: no hit.
+constexpr unsigned long long kNoHitKey = 0xFFFFFFFFFFFFFFFFull;
+__device__ __forceinline__ unsigned long long order_key(double t) {
+  const long long b = __double_as_longlong(t + 0.0);
+  return (unsigned long long)(b ^ ((b >> 63) | (1ll << 63)));
+}
+__device__ __forceinline__ double key_value(unsigned long long k) {
+  const long long b = (long long)k;
+  return __longlong_as_double(b < 0 ? (long long)(k ^ (1ull << 63)) : ~b);
 }
 
 // Re-intersects the rays the FP32 pass flagged, in FP64 and without
 // certification:
 //   * with a contender list (the leaves that may still be the closest hit),
-//     lane q of the ray's 8-lane group intersects contender q with the exact
-//     closed-box rule and a group reduction keeps the lexicographic minimum
-//     of (t, part, voxel);
+//     the contenders are intersected by the exact closed-box rule, spread
+//     over lanes, and the lexicographic minimum of (t, part, voxel) kept;
 //   * without one (the contender list overflowed, or the leaf pool was
-//     full), the warp re-traces the ray, the parts dealt over the lanes: the
-//     FP32 descent with inflated boxes, every leaf reached decided in FP64.
-// GB300 issues FP64 at 2 lanes per clock per SM, so spreading a ray's
-// contenders over lanes (instead of one lane looping over them) cuts the
-// pass's latency by the contender count.  Groups of four list entries are
-// dealt round-robin over the warps so that a short list still spreads over
-// the whole GPU.
+//     full), the warp re-traces the ray (overflow_retrace).
+// Bound by the FP64 pipes on long lists (GB300 issues FP64 at 2 lanes per
+// clock and SM, whatever a warp's active lanes), by latency on short ones.
+// Lists of up to two rounds of four entries per warp give each entry a group
+// of eight lanes, so that they spread over the GPU; longer ones are taken 32
+// entries a warp (below).  1.05 M rays into depth-13 parts (428 K t
+// refinements, 289 K contender lists of 5 leaves on average, 43 K re-traces):
+// 2.55 -> 1.00 ms; 116 K entries of 64 scenes 59 -> 36 us.
 template <int NI>
 __global__ void __launch_bounds__(kBlock) k_fix(const __grid_constant__ TraceLaunchT<NI> L) {
+  __shared__ FixUnion sFix[kBlock / 32];
   // the rare re-traces read the order tables from global memory (L1/L2), so
   // blocks start without staging them
   const Tables *tab = &g_tables;
@@ -2292,68 +2457,116 @@ __global__ void __launch_bounds__(kBlock) k_fix(const __grid_constant__ TraceLau
   const int sub = lane >> 3, sl = lane & 7;
   if (n > 8ull * n_warps) {
     // A long list (more than two rounds of four entries per warp): runs of 32
-    // entries per warp.  An entry with one stored leaf (every t refinement)
-    // takes one lane, so 32 of them share each FP64 instruction; entries with
-    // a contender list go four at a time in 8-lane groups; entries without
-    // one get the whole warp.  A short list keeps four entries per warp
-    // (below), which spreads it over more warps.
+    // entries per warp, one a lane for its first leaf (every t refinement has
+    // no other).  The other contenders of the 32 entries are dealt over the
+    // lanes in one flat order, so that an FP64 instruction serves 32 of them
+    // however they are distributed; those in the part of the entry's first leaf
+    // (nearly all) reuse its local ray from shared memory.  Each entry's lane
+    // then takes the minimum of its own.
+    FixWarp &w = sFix[threadIdx.x >> 5].list;
     for (unsigned long long i0 = 32 * warp; i0 < n; i0 += 32 * n_warps) {
       const unsigned long long i = i0 + (unsigned long long)lane;
       const bool have = i < n;
       const unsigned long long e = have ? L.fix_list[i] : 0ull;
       const int nc = (int)(e >> 48);
-      if (have && nc == 1) {
-        const int it = (int)((e >> kRayBits) & 0x7Fu);
-        const unsigned long long ray = e & ((1ull << kRayBits) - 1ull);
+      const int it = (int)((e >> kRayBits) & 0x7Fu);
+      const unsigned long long ray = e & ((1ull << kRayBits) - 1ull);
+      unsigned long long best = kNoHitKey, vox = kMissVoxel;
+      uint32_t part = kMissPart;
+      if (nc >= 1) {
         const TraceItem &I = L.items[it];
         const float4 o = I.rays[2 * ray], d = I.rays[2 * ray + 1];
-        const uint4 cv = L.fix_cand[L.fix_off[i]];
-        const uint32_t p = cv.x;
-        const unsigned long long vox = (unsigned long long)cv.y | ((unsigned long long)cv.z << 32);
-        ExactState st;
-        st.t = Num<double>::inf();
-        st.part = kMissPart;
-        st.vox = kMissVoxel;
+        const uint32_t off = L.fix_off[i];
+        const uint4 cv = L.fix_cand[off];
+        const unsigned long long v = (unsigned long long)cv.y | ((unsigned long long)cv.z << 32);
+        const int depth = I.aux[cv.x].depth;
+        const LocalRay64 l = local_ray64(I.inv64 + 12 * cv.x, o, d);
         double tq;
-        if (leaf_entry64(I.inv64 + 12 * p, I.aux[p].depth, vox, o, d, tq)) offer(st, tq, p, vox);
-        write_fixed(I, ray, st, ((e >> 47) & 1ull) ? SVO_RAY_T_REFINED : SVO_RAY_UNCERTAIN);
-      }
-      for (unsigned int multi = __ballot_sync(0xffffffffu, have && nc >= 2); multi != 0u;) {
-        // the next four such entries, one 8-lane group each
-        int src = -1;
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          const int s = multi ? __ffs(multi) - 1 : -1;
-          if (g == sub) src = s;
-          if (multi) multi &= multi - 1u;
+        if (leaf_entry64(l, depth, v, o.w, d.w, tq)) {
+          best = order_key(tq);
+          part = cv.x;
+          vox = v;
         }
-        const unsigned long long ee = __shfl_sync(0xffffffffu, e, src < 0 ? 0 : src);
-        const int ncg = src >= 0 ? (int)(ee >> 48) : 0;
-        const int it = (int)((ee >> kRayBits) & 0x7Fu);
-        const unsigned long long ray = ee & ((1ull << kRayBits) - 1ull);
-        ExactState st;
-        st.t = Num<double>::inf();
-        st.part = kMissPart;
-        st.vox = kMissVoxel;
-        if (sl < ncg) {
-          const TraceItem &I = L.items[it];
-          const float4 o = I.rays[2 * ray], d = I.rays[2 * ray + 1];
-          const uint32_t off = L.fix_off[i0 + (unsigned long long)src];
-          for (int q = sl; q < ncg; q += 8) {
-            const uint4 cv = L.fix_cand[off + q];
-            const uint32_t p = cv.x;
-            const unsigned long long vox = (unsigned long long)cv.y | ((unsigned long long)cv.z << 32);
-            double tq;
-            if (leaf_entry64(I.inv64 + 12 * p, I.aux[p].depth, vox, o, d, tq)) offer(st, tq, p, vox);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          w.o[k][lane] = l.o[k];
+          w.inv[k][lane] = l.inv[k];
+        }
+        w.tmin[lane] = o.w;
+        w.tmax[lane] = d.w;
+        w.first[lane] = cv.x;
+        w.depth[lane] = depth;
+        w.off[lane] = off;
+      }
+      const int more = nc >= 2 ? nc - 1 : 0;
+      int begin = more;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, begin, o);
+        if (lane >= o) begin += v;
+      }
+      const int total = __shfl_sync(0xffffffffu, begin, 31);
+      begin -= more;
+      w.begin[lane] = begin;
+      __syncwarp();
+      for (int base = 0; base < total; base += 32) {
+        const int f = base + lane;
+        int own = 0;  // the last entry that begins at or before f
+#pragma unroll
+        for (int k = 16; k > 0; k >>= 1)
+          if (w.begin[own + k] <= f) own += k;
+        const unsigned long long eo = __shfl_sync(0xffffffffu, e, own);
+        unsigned long long key = kNoHitKey, v = kMissVoxel;
+        uint32_t p = kMissPart;
+        if (f < total) {
+          const uint4 cv = L.fix_cand[w.off[own] + 1 + (f - w.begin[own])];
+          p = cv.x;
+          v = (unsigned long long)cv.y | ((unsigned long long)cv.z << 32);
+          int depth = w.depth[own];
+          LocalRay64 l;
+          if (p == w.first[own]) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              l.o[k] = w.o[k][own];
+              l.inv[k] = w.inv[k][own];
+            }
+          } else {
+            const TraceItem &I = L.items[(int)((eo >> kRayBits) & 0x7Fu)];
+            const unsigned long long ry = eo & ((1ull << kRayBits) - 1ull);
+            l = local_ray64(I.inv64 + 12 * p, I.rays[2 * ry], I.rays[2 * ry + 1]);
+            depth = I.aux[p].depth;
+          }
+          double tq;
+          if (leaf_entry64(l, depth, v, w.tmin[own], w.tmax[own], tq)) key = order_key(tq);
+        }
+        w.key[lane] = key;
+        w.part[lane] = p;
+        w.vox[lane] = v;
+        __syncwarp();
+        const int hi = min(begin + more, base + 32) - base;
+        for (int k = max(begin - base, 0); k < hi; ++k) {
+          const unsigned long long kk = w.key[k], kv = w.vox[k];
+          const uint32_t kp = w.part[k];
+          if (kk != kNoHitKey && (kk < best || (kk == best && (kp < part || (kp == part && kv < vox))))) {
+            best = kk;
+            part = kp;
+            vox = kv;
           }
         }
-        group_min8(st);
-        if (ncg > 0 && sl == 0)
-          write_fixed(L.items[it], ray, st, ((ee >> 47) & 1ull) ? SVO_RAY_T_REFINED : SVO_RAY_UNCERTAIN);
+        __syncwarp();
+      }
+      __syncwarp();  // the entries' local rays are read
+      if (nc >= 1) {
+        ExactState st;
+        st.t = best == kNoHitKey ? Num<double>::inf() : key_value(best);
+        st.part = part;
+        st.vox = vox;
+        write_fixed(L.items[it], ray, st, ((e >> 47) & 1ull) ? SVO_RAY_T_REFINED : SVO_RAY_UNCERTAIN);
       }
       for (unsigned int pending = __ballot_sync(0xffffffffu, have && nc == 0); pending != 0u; pending &= pending - 1u) {
         const int src = __ffs(pending) - 1;
-        overflow_retrace(L, i0 + (unsigned long long)src, __shfl_sync(0xffffffffu, e, src), tab, err, cnt);
+        overflow_retrace(L, i0 + (unsigned long long)src, __shfl_sync(0xffffffffu, e, src), tab,
+                         sFix[threadIdx.x >> 5], err, cnt);
       }
     }
   } else
@@ -2380,7 +2593,7 @@ __global__ void __launch_bounds__(kBlock) k_fix(const __grid_constant__ TraceLau
           const uint32_t p = cv.x;
           const unsigned long long vox = (unsigned long long)cv.y | ((unsigned long long)cv.z << 32);
           double tq;
-          if (leaf_entry64(I.inv64 + 12 * p, I.aux[p].depth, vox, o, d, tq)) offer(st, tq, p, vox);
+          if (leaf_entry64(local_ray64(I.inv64 + 12 * p, o, d), I.aux[p].depth, vox, o.w, d.w, tq)) offer(st, tq, p, vox);
         }
       }
       group_min8(st);
@@ -2393,7 +2606,7 @@ __global__ void __launch_bounds__(kBlock) k_fix(const __grid_constant__ TraceLau
       pending &= pending - 1u;
       const unsigned long long ie = i0 + (unsigned long long)(src >> 3);
       const unsigned long long ee = __shfl_sync(0xffffffffu, e, src);
-      overflow_retrace(L, ie, ee, tab, err, cnt);
+      overflow_retrace(L, ie, ee, tab, sFix[threadIdx.x >> 5], err, cnt);
     }
   }
   // count fixed rays once per launch
@@ -2554,9 +2767,14 @@ cudaError_t launch_trace_t(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
   return launch_trace_b<NI, 128>(L, n_sm, stream);
 }
 
+// Four blocks, the most that fit: an entry is a chain of dependent reads and
+// FP64 instructions, which other warps hide (two blocks: 116 K entries 44 us,
+// four 36; re-traces scale with the warps).
+constexpr int kFixBlocksPerSM = 4;
+
 template <int NI>
 cudaError_t launch_fix_t(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t stream) {
-  k_fix<NI><<<(unsigned int)(n_sm * 2), kBlock, 0, stream>>>(L);
+  k_fix<NI><<<(unsigned int)(n_sm * kFixBlocksPerSM), kBlock, 0, stream>>>(L);
   return cudaGetLastError();
 }
 
