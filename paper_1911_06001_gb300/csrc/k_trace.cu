@@ -75,6 +75,7 @@ struct TraceLaunchT {
   unsigned long long *queue_tile;   // SVO_TRACE_WAVEFRONT: tile counter of the descent launch
   TileEntry *tiles;                 // tile-culled image trace: the tiles to trace
   unsigned int *tile_count;         // their number
+  unsigned long long *clean;        // the FP64 pass leaves these kCounterWords at zero, and every dirty flag (nullptr: no)
 };
 
 namespace {
@@ -94,6 +95,14 @@ constexpr int kTraceThreadsPerSM = 768;
 // it runs only tiles that descend (nine requests, 6.7 M rays: 0.707 ms, 0.691
 // at 20 warps; 2.1 M rays against 1024 parts: 0.249 and 0.245).
 constexpr int kListThreadsPerSM = 512;
+
+// Programmatic dependent launches: the kernels of the chain culling -> trace
+// -> FP64 pass are launched while the one before still runs (launch_after),
+// do what does not depend on it, and wait for all of it here.  None asks for
+// its successor to start early: the successor's blocks would only wait, in
+// registers and shared memory that other streams' kernels can use (eight
+// views of three graphs at a time: 103 us a graph, 119 with early starts).
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 constexpr unsigned long long kRayBits = 40;
 constexpr uint32_t kNoCand = 0xFFFFFFFFu;  // a list slot without stored leaves
@@ -1518,6 +1527,7 @@ __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? 
   uint32_t *sMbox = reinterpret_cast<uint32_t *>(sTop + ntop_all) + threadIdx.x;  // word-major, stride BLOCK
   const uint32_t sTopAddr = (uint32_t)__cvta_generic_to_shared(sTop);
   load_tables(tab);
+  wait_for_previous();
   if (L.one_scene) {
     const TraceItem &I0 = L.items[0];
     for (int i = threadIdx.x; i < I0.n_parts; i += BLOCK) {
@@ -1760,6 +1770,7 @@ __global__ void __launch_bounds__(kCullThreads, kCullThreadsPerSM / kCullThreads
   Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
   uint32_t n_rays = 0;
   const int lane = threadIdx.x & 31;
+  wait_for_previous();
   int staged = -1;
   CullTables t = {nullptr, nullptr, nullptr, nullptr, nullptr};
   if (L.same_scene && L.n_items == 1) {
@@ -1869,6 +1880,7 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_cull(const __grid_constan
   const int lane = threadIdx.x & 31;
   const unsigned int below = (1u << lane) - 1u;
   uint16_t *list = sList[threadIdx.x >> 5];
+  wait_for_previous();
   const unsigned long long n_warps = (unsigned long long)gridDim.x * (kTileThreads / 32);
   for (unsigned long long tile = (unsigned long long)blockIdx.x * (kTileThreads / 32) + (threadIdx.x >> 5);
        tile < L.n_tiles; tile += n_warps) {
@@ -1983,6 +1995,7 @@ __global__ void __launch_bounds__(BLOCK, 512 / BLOCK) k_descend(const __grid_con
   Cluster *sCl = reinterpret_cast<Cluster *>(sAux + sp);
   int32_t *sOrd = reinterpret_cast<int32_t *>(sCl + sc);
   load_tables(tab);
+  wait_for_previous();
   if (L.one_scene) {
     const TraceItem &I0 = L.items[0];
     for (int i = threadIdx.x; i < I0.n_parts; i += BLOCK) {
@@ -2444,6 +2457,7 @@ __global__ void __launch_bounds__(kBlock) k_fix(const __grid_constant__ TraceLau
   const Tables *tab = &g_tables;
   unsigned int err = 0;
   Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
+  wait_for_previous();
   const unsigned long long n = min((unsigned long long)*L.fix_count, L.fix_capacity);
   const int lane = threadIdx.x & 31;
   const unsigned long long n_warps = (unsigned long long)gridDim.x * (blockDim.x / 32);
@@ -2609,6 +2623,22 @@ __global__ void __launch_bounds__(kBlock) k_fix(const __grid_constant__ TraceLau
       overflow_retrace(L, ie, ee, tab, sFix[threadIdx.x >> 5], err, cnt);
     }
   }
+  if (L.clean) {
+    // Pose changes are tracked relative to a scene's latest trace, and the next
+    // trace expects its counters at zero: left so here, by the last block to
+    // come through, instead of by memsets around the launches (two per call and
+    // one per scene of a batch, each about as long as an empty kernel).
+    for (int i = blockIdx.x; i < L.n_items; i += gridDim.x) {
+      uint8_t *dirty = const_cast<uint8_t *>(L.items[i].dirty);
+      for (int p = threadIdx.x; p < L.items[i].n_parts; p += kBlock) dirty[p] = 0;
+    }
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&L.clean[kCounterWords - 1], 1ull) == gridDim.x - 1;
+    __syncthreads();
+    if (last)
+      for (int k = threadIdx.x; k < (int)kCounterWords; k += kBlock) L.clean[k] = 0ull;
+  }
   // count fixed rays once per launch
   if (L.stats && blockIdx.x == 0 && threadIdx.x == 0 && (L.flags & SVO_TRACE_STATS)) atomicAdd(&L.stats->fixed, n);
   if (err) atomicOr(L.err, err);
@@ -2668,6 +2698,22 @@ cudaError_t blocks_per_sm(K kern, int block, size_t smem, int &per_sm) {
   return cudaSuccess;
 }
 
+// Launches a kernel that waits for the one before it by itself.
+template <typename T>
+cudaError_t launch_after(void (*kern)(T), unsigned int grid, int block, size_t smem, cudaStream_t stream, const T &L) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3((unsigned int)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, L);
+}
+
 template <int NI, int BLOCK>
 cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t stream) {
   const bool stats = (L.flags & SVO_TRACE_STATS) && L.stats;
@@ -2700,8 +2746,7 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
     const unsigned long long need = (L.n_tiles + kCullWarps - 1) / kCullWarps;
     if (grid > need) grid = need;
     if (grid == 0) return cudaSuccess;
-    ck<<<(unsigned int)grid, kCullThreads, csmem, stream>>>(L);
-    e = cudaGetLastError();
+    e = launch_after(ck, (unsigned int)grid, kCullThreads, csmem, stream, L);
     if (e != cudaSuccess) return e;
     // the number of queued rays is known on the device only: a full persistent grid
     const size_t smem = trace_smem_bytes(L.stack_levels, parts, clusters, BLOCK, 0, 0);
@@ -2709,8 +2754,7 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
     e = blocks_per_sm(kq, BLOCK, smem, per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    kq<<<(unsigned int)(n_sm * per_sm), BLOCK, smem, stream>>>(L);
-    return cudaGetLastError();
+    return launch_after(kq, (unsigned int)(n_sm * per_sm), BLOCK, smem, stream, L);
   }
   if (L.tiles) {
     // an image trace: the tile-culling launch, then the trace of the tiles it queued
@@ -2721,8 +2765,7 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
     const unsigned long long cull_blocks = (L.n_tiles + kTileThreads / 32 - 1) / (kTileThreads / 32);
     if (grid > cull_blocks) grid = cull_blocks;
     if (grid == 0) return cudaSuccess;
-    k_tile_cull<NI><<<(unsigned int)grid, kTileThreads, 0, stream>>>(L);
-    e = cudaGetLastError();
+    e = launch_after(k_tile_cull<NI>, (unsigned int)grid, kTileThreads, 0, stream, L);
     if (e != cudaSuccess) return e;
     const size_t smem = trace_smem_bytes(L.stack_levels, L.one_scene ? L.items[0].n_parts : 0,
                                          L.one_scene ? L.items[0].n_clusters : 0, BLOCK, 0, 0);
@@ -2733,8 +2776,7 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
     grid = (unsigned long long)n_sm * (per_sm < 1 ? 1 : per_sm);
     const unsigned long long blocks = (L.n_tiles + BLOCK / 32 - 1) / (BLOCK / 32);
     if (grid > blocks) grid = blocks;
-    kl<<<(unsigned int)grid, BLOCK, smem, stream>>>(L);
-    return cudaGetLastError();
+    return launch_after(kl, (unsigned int)grid, BLOCK, smem, stream, L);
   }
   // the staged top levels only in the common kernel (counting, reuse and grid traces give the same
   // results without them)
@@ -2756,8 +2798,7 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
   const unsigned long long need = (L.n_tiles + BLOCK / 32 - 1) / (BLOCK / 32);
   if (grid > need) grid = need;
   if (grid == 0) return cudaSuccess;
-  kern<<<(unsigned int)grid, BLOCK, smem, stream>>>(L);
-  return cudaGetLastError();
+  return launch_after(kern, (unsigned int)grid, BLOCK, smem, stream, L);
 }
 
 template <int NI>
@@ -2774,8 +2815,7 @@ constexpr int kFixBlocksPerSM = 4;
 
 template <int NI>
 cudaError_t launch_fix_t(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t stream) {
-  k_fix<NI><<<(unsigned int)(n_sm * kFixBlocksPerSM), kBlock, 0, stream>>>(L);
-  return cudaGetLastError();
+  return launch_after(k_fix<NI>, (unsigned int)(n_sm * kFixBlocksPerSM), kBlock, 0, stream, L);
 }
 
 template <int NI>
@@ -2816,6 +2856,7 @@ void fill_launch(const TraceLaunch &src, TraceLaunchT<NI> &dst) {
   dst.queue_tile = src.queue_tile;
   dst.tiles = src.tiles;
   dst.tile_count = src.tile_count;
+  dst.clean = src.clean;
 }
 
 }  // namespace

@@ -94,13 +94,15 @@ constexpr int kTileCullParts = 20;
 // ones that need more are traced in one launch).
 inline unsigned long long tile_capacity(unsigned long long cap) { return cap / 16; }
 
-constexpr size_t kCounterWords = kQueueCountWords + kMaxBatchItems / 2;
-
 // Scratch of one stream: launch counters and the FP64 re-intersection list.
 struct Slot {
-  // [0] tile counter, [1] fix count (low 32 bits), [2] pool count, [3] tile counter of the wavefront
-  // descent launch, then kMaxBatchItems 32-bit queue counts
+  // [0] tile counter, [1] fix count and queued image tiles (32 bits each), [2] pool count, [3] tile
+  // counter of the wavefront descent launch, then kMaxBatchItems 32-bit queue counts and the FP64 pass's
+  // blocks done.  Two sets.  The first is at zero between calls: a call that runs the FP64 pass has it
+  // cleared there, any other clears it at its end.  The second belongs to a deferred FP64 pass, which reads
+  // it later, and is cleared at the start of each such call.
   unsigned long long *d_counters = nullptr;
+  bool counters_lost = false;  // a launch failed half-way: the first set is cleared before the next call
   unsigned long long *d_fix = nullptr;
   unsigned long long cap = 0;
   uint4 *d_cand = nullptr;                   // pool of leaves stored for the FP64 pass
@@ -177,7 +179,16 @@ AssetRec *find_asset(svo_ctx *ctx, svo_handle h) {
 svo_status get_slot(svo_ctx *ctx, void *stream, unsigned long long need, Slot **out) {
   std::lock_guard<std::mutex> g(ctx->mu);
   Slot &s = ctx->slots[stream];
-  if (!s.d_counters) CK(cudaMalloc(&s.d_counters, kCounterWords * sizeof(unsigned long long)));
+  if (!s.d_counters) {
+    unsigned long long *p = nullptr;
+    CK(cudaMalloc(&p, 2 * kCounterWords * sizeof(unsigned long long)));
+    const cudaError_t e = cudaMemsetAsync(p, 0, 2 * kCounterWords * sizeof(unsigned long long), (cudaStream_t)stream);
+    if (e != cudaSuccess) {
+      cudaFree(p);
+      return fail(SVO_ERR_CUDA, "launch counters: %s", cudaGetErrorString(e));
+    }
+    s.d_counters = p;
+  }
   if (need > s.cap) {
     unsigned long long cap = need < 65536 ? 65536 : need;
     unsigned long long *p = nullptr;
@@ -333,6 +344,8 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
   Slot *slot = nullptr;
   svo_status rc = get_slot(ctx, stream, total_rays, &slot);
   if (rc != SVO_OK) return rc;
+  const bool fix = (L.flags & SVO_TRACE_FP64_FIX) != 0, defer = fix && (L.flags & SVO_TRACE_DEFER_FIX);
+  unsigned long long *const counters = slot->d_counters + (defer ? kCounterWords : 0);
   const int order_mode = (L.flags & SVO_TRACE_ORDER_ORIGIN) ? 2 : ((L.flags & SVO_TRACE_ORDER_DIR) ? 1 : 0);
   if (order_mode) {
     size_t need = 0;
@@ -385,7 +398,7 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
   // link (the tiles that go on would be read twice: 250,000 mapped rays take
   // 201 us in one launch, 221 in two).
   L.tiles = nullptr;
-  L.tile_count = reinterpret_cast<unsigned int *>(slot->d_counters + 1) + 1;
+  L.tile_count = reinterpret_cast<unsigned int *>(counters + 1) + 1;
   if (!wave && !host_rays && ctx->rays_per_lane == 1 && ctx->smem_levels == 0 && !(L.flags & SVO_TRACE_STATS) &&
       (L.flags & (SVO_TRACE_CULL | SVO_TRACE_SORT)) == (SVO_TRACE_CULL | SVO_TRACE_SORT)) {
     unsigned long long image_tiles = 0;
@@ -400,8 +413,8 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
       L.tiles = slot->d_tiles;
   }
   L.queue = nullptr;
-  L.queue_count = reinterpret_cast<unsigned int *>(slot->d_counters + kQueueCountWords);
-  L.queue_tile = slot->d_counters + 3;
+  L.queue_count = reinterpret_cast<unsigned int *>(counters + kQueueCountWords);
+  L.queue_tile = counters + 3;
   if (wave) {
     if (total_rays > slot->queue_cap) {
       std::lock_guard<std::mutex> g(ctx->mu);
@@ -422,22 +435,23 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
       q += L.items[i].n;
     }
   }
-  L.tile_counter = slot->d_counters;
-  L.fix_count = reinterpret_cast<unsigned int *>(slot->d_counters + 1);
+  L.tile_counter = counters;
+  L.fix_count = reinterpret_cast<unsigned int *>(counters + 1);
   L.fix_list = slot->d_fix;
   L.fix_capacity = slot->cap;
   L.fix_cand = slot->d_cand;
   L.cand_capacity = slot->cand_cap;
-  L.cand_count = reinterpret_cast<unsigned int *>(slot->d_counters + 2);
+  L.cand_count = reinterpret_cast<unsigned int *>(counters + 2);
   L.fix_off = slot->d_off;
   L.err = ctx->d_err;
   L.block = ctx->block;
   L.rays_per_lane = ctx->rays_per_lane;
   set_top_levels(ctx, only, L);
-  CK(cudaMemsetAsync(slot->d_counters, 0,
-                     wave ? kQueueCountWords * sizeof(unsigned long long) + (size_t)L.n_items * sizeof(unsigned int)
-                          : 3 * sizeof(unsigned long long),
-                     st));
+  L.clean = fix && !defer ? counters : nullptr;
+  if (defer || slot->counters_lost) {
+    CK(cudaMemsetAsync(counters, 0, kCounterWords * sizeof(unsigned long long), st));
+    if (!defer) slot->counters_lost = false;
+  }
   // the scene grids this launch walks: SVO_TRACE_GRID's from
   // kGridWalkMinParts parts on, and those its culling launch uses
   unsigned long long tests = 0;
@@ -453,20 +467,28 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
     GridLaunch gl;
     if (grid_jobs(L.items, L.n_items, gl) > 0) CK(launch_grid(gl, st));
   }
-  CK(launch_trace(L, ctx->n_sm, st));
-  // pose changes are tracked relative to each scene's latest trace
-  for (int i = 0; i < L.n_items; ++i) {
-    bool seen = false;
-    for (int j = 0; j < i; ++j) seen = seen || L.items[j].dirty == L.items[i].dirty;
-    if (!seen) CK(cudaMemsetAsync(const_cast<uint8_t *>(L.items[i].dirty), 0, (size_t)L.items[i].n_parts, st));
-  }
+  cudaError_t e = launch_trace(L, ctx->n_sm, st);
   delete slot->pending;
   slot->pending = nullptr;
-  if (L.flags & SVO_TRACE_FP64_FIX) {
-    if (L.flags & SVO_TRACE_DEFER_FIX)
-      slot->pending = new TraceLaunch(L);
-    else
-      CK(launch_fix(L, ctx->n_sm, st));
+  if (L.clean) {
+    if (e == cudaSuccess) e = launch_fix(L, ctx->n_sm, st);
+  } else {
+    // pose changes are tracked relative to each scene's latest trace
+    for (int i = 0; i < L.n_items && e == cudaSuccess; ++i) {
+      bool seen = false;
+      for (int j = 0; j < i; ++j) seen = seen || L.items[j].dirty == L.items[i].dirty;
+      if (!seen) e = cudaMemsetAsync(const_cast<uint8_t *>(L.items[i].dirty), 0, (size_t)L.items[i].n_parts, st);
+    }
+    if (e == cudaSuccess) {
+      if (defer)
+        slot->pending = new TraceLaunch(L);
+      else
+        e = cudaMemsetAsync(counters, 0, kCounterWords * sizeof(unsigned long long), st);
+    }
+  }
+  if (e != cudaSuccess) {
+    slot->counters_lost = true;
+    return fail(SVO_ERR_CUDA, "trace: %s", cudaGetErrorString(e));
   }
   return SVO_OK;
 }

@@ -146,6 +146,8 @@ static_assert(sizeof(TileEntry) == 64, "TileEntry is 64 bytes");
 constexpr uint32_t kTileOpen = 0xFFFFFFFFu;
 
 constexpr int kQueueCountWords = 4;  // per-stream counters before the per-item queue counts (64-bit words)
+// One set of launch counters: kQueueCountWords, kMaxBatchItems 32-bit queue counts, and the FP64 pass's blocks done.
+constexpr size_t kCounterWords = kQueueCountWords + kMaxBatchItems / 2 + 1;
 
 // Warp tiles of every item, laid out one item after another: sets each
 // item's tile_begin (and tiles_x) and returns the total.  A tile is
@@ -199,6 +201,7 @@ struct TraceLaunch {
   unsigned long long *queue_tile;     // SVO_TRACE_WAVEFRONT: tile counter of the descent launch; zeroed
   TileEntry *tiles;                   // tile-culled image trace: the tiles to trace (nullptr: one launch over all)
   unsigned int *tile_count;           // their number; zeroed
+  unsigned long long *clean;          // counters the FP64 pass leaves at zero, with every dirty flag (nullptr: no)
 };
 
 // Kernel launchers (k_trace.cu, k_refit.cu).
