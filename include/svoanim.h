@@ -336,7 +336,9 @@ svo_status trace_rays(svo_scene *scene, const float *rays, uint64_t n, svo_hit *
                       uint32_t flags, svo_trace_stats *stats, void *stream);
 /* (With SVO_TRACE_ORDER_DIR / _ORIGIN the rays are first counting-sorted by a
  * 14-bit direction / origin-cell key into per-stream scratch, grown like the
- * FP64 list; hits still land at each ray's own index.) */
+ * FP64 list; hits still land at each ray's own index.  trace_rays with _ORIGIN
+ * takes the wavefront shape instead where its flags allow it, with that
+ * shape's queue as scratch, and sorts where the queue finds no room.) */
 /* Batched trace: every item's rays against its own scene, in one persistent
  * launch whose thread blocks take fixed-size tiles of rays from a device work
  * counter (async), or -- with SVO_TRACE_WAVEFRONT -- in a culling launch and a

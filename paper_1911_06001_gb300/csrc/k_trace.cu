@@ -75,6 +75,7 @@ struct TraceLaunchT {
   unsigned long long *queue_tile;   // SVO_TRACE_WAVEFRONT: tile counter of the descent launch
   TileEntry *tiles;                 // tile-culled image trace: the tiles to trace
   unsigned int *tile_count;         // their number
+  unsigned long long gate;          // see TraceLaunch
   unsigned long long *clean;        // the FP64 pass leaves these kCounterWords at zero, and every dirty flag (nullptr: no)
 };
 
@@ -1528,6 +1529,7 @@ __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? 
   const uint32_t sTopAddr = (uint32_t)__cvta_generic_to_shared(sTop);
   load_tables(tab);
   wait_for_previous();
+  if (L.gate && *L.queue_count < L.gate) return;  // the descent launch has the queued rays
   if (L.one_scene) {
     const TraceItem &I0 = L.items[0];
     for (int i = threadIdx.x; i < I0.n_parts; i += BLOCK) {
@@ -1996,6 +1998,7 @@ __global__ void __launch_bounds__(BLOCK, 512 / BLOCK) k_descend(const __grid_con
   int32_t *sOrd = reinterpret_cast<int32_t *>(sCl + sc);
   load_tables(tab);
   wait_for_previous();
+  if (L.gate && *L.queue_count >= L.gate) return;  // the single launch traces every ray
   if (L.one_scene) {
     const TraceItem &I0 = L.items[0];
     for (int i = threadIdx.x; i < I0.n_parts; i += BLOCK) {
@@ -2754,7 +2757,17 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
     e = blocks_per_sm(kq, BLOCK, smem, per_sm);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    return launch_after(kq, (unsigned int)(n_sm * per_sm), BLOCK, smem, stream, L);
+    e = launch_after(kq, (unsigned int)(n_sm * per_sm), BLOCK, smem, stream, L);
+    if constexpr (NI == 1) {
+      if (e != cudaSuccess || !L.gate) return e;
+      TraceLaunchT<NI> G = L;
+      G.tile_counter = L.queue_tile;  // the culling launch has used the other, and only one of these two claims from it
+      auto kg = k_trace<NI, false, BLOCK, false, false>;
+      e = blocks_per_sm(kg, BLOCK, smem, per_sm);
+      if (e != cudaSuccess) return e;
+      return launch_after(kg, (unsigned int)(n_sm * (per_sm < 1 ? 1 : per_sm)), BLOCK, smem, stream, G);
+    }
+    return e;
   }
   if (L.tiles) {
     // an image trace: the tile-culling launch, then the trace of the tiles it queued
@@ -2856,6 +2869,7 @@ void fill_launch(const TraceLaunch &src, TraceLaunchT<NI> &dst) {
   dst.queue_tile = src.queue_tile;
   dst.tiles = src.tiles;
   dst.tile_count = src.tile_count;
+  dst.gate = src.gate;
   dst.clean = src.clean;
 }
 

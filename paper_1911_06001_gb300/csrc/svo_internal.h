@@ -201,6 +201,7 @@ struct TraceLaunch {
   unsigned long long *queue_tile;     // SVO_TRACE_WAVEFRONT: tile counter of the descent launch; zeroed
   TileEntry *tiles;                   // tile-culled image trace: the tiles to trace (nullptr: one launch over all)
   unsigned int *tile_count;           // their number; zeroed
+  unsigned long long gate;            // wavefront: from this many queued rays on the single launch traces them all (0: never)
   unsigned long long *clean;          // counters the FP64 pass leaves at zero, with every dirty flag (nullptr: no)
 };
 
