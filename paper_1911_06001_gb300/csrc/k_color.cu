@@ -177,7 +177,7 @@ __device__ __forceinline__ bool shade_fast(uint32_t color, float t, float4 o, fl
 
 // One thread per pixel.  Bound by the FP64 pipes: with every decision in FP64
 // (two matrix products, three divisions, a square root and a channel each
-// about seven instructions) 0.16 M hits of 0.98 M pixels took 57 us, now 26.
+// about seven instructions) 0.16 M hits of 0.98 M pixels took 57 us, now 28.
 __global__ void k_shade(const float4 *__restrict__ rays, const uint4 *__restrict__ hits, unsigned long long n,
                         const PartStatic *__restrict__ stat, const double *__restrict__ inv64, int n_parts,
                         const __grid_constant__ ShadeArgs sa, uint32_t *__restrict__ rgb) {

@@ -96,6 +96,11 @@ constexpr int kTraceThreadsPerSM = 768;
 // it runs only tiles that descend (nine requests, 6.7 M rays: 0.707 ms, 0.691
 // at 20 warps; 2.1 M rays against 1024 parts: 0.249 and 0.245).
 constexpr int kListThreadsPerSM = 512;
+// Image tiles in one launch keep 16 warps as well: their coherent lanes fill
+// the issue slots, and 128 registers do without spills.  24 / 20 / 16 warps: a
+// 1920x1080 frame of a 16-part figure 0.158 / 0.153 / 0.151 ms alone and 183 /
+// 175 / 165 us a call with others behind it.
+constexpr int kImageThreadsPerSM = 512;
 
 // Programmatic dependent launches: the kernels of the chain culling -> trace
 // -> FP64 pass are launched while the one before still runs (launch_after),
@@ -1511,8 +1516,9 @@ __device__ __forceinline__ void finish_ray(const TraceLaunchT<NI> &L, const Trac
 // instantiation: the staged-node base is one more live register, which the
 // common kernel does not carry).
 // LIST: only the image tiles k_tile_cull queued, each with its parts.
-template <int NI, bool STATS, int BLOCK, bool REUSE, bool GRID, bool TOP = false, bool LIST = false>
-__global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? kListThreadsPerSM : kTraceThreadsPerSM) / BLOCK) k_trace(const __grid_constant__ TraceLaunchT<NI> L) {
+// IMAGE: every item's rays are image tiles (the same code at more registers).
+template <int NI, bool STATS, int BLOCK, bool REUSE, bool GRID, bool TOP = false, bool LIST = false, bool IMAGE = false>
+__global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? kListThreadsPerSM : IMAGE ? kImageThreadsPerSM : kTraceThreadsPerSM) / BLOCK) k_trace(const __grid_constant__ TraceLaunchT<NI> L) {
   extern __shared__ __align__(16) unsigned char smem[];
   // [tables | traversal stacks, level-major | staged part tables]
   Tables *tab = reinterpret_cast<Tables *>(smem);
@@ -2794,6 +2800,8 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
   // the staged top levels only in the common kernel (counting, reuse and grid traces give the same
   // results without them)
   const bool top = L.one_scene && L.top_nodes > 0 && !stats && !reuse && !walk;
+  bool image = true;
+  for (int i = 0; i < L.n_items; ++i) image = image && L.items[i].tiles_x != 0;
   const size_t smem = trace_smem_bytes(L.stack_levels, L.one_scene ? L.items[0].n_parts : 0,
                                        L.one_scene ? L.items[0].n_clusters : 0, BLOCK, walk ? L.mbox_words : 0,
                                        top ? L.top_nodes : 0);
@@ -2801,6 +2809,7 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
               : stats ? (reuse ? k_trace<NI, true, BLOCK, true, false> : k_trace<NI, true, BLOCK, false, false>)
               : reuse ? k_trace<NI, false, BLOCK, true, false>
               : top   ? k_trace<NI, false, BLOCK, false, false, true>
+              : image ? k_trace<NI, false, BLOCK, false, false, false, false, true>
                       : k_trace<NI, false, BLOCK, false, false>;
   int per_sm = 0;
   const cudaError_t e = blocks_per_sm(kern, BLOCK, smem, per_sm);
