@@ -167,41 +167,41 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
       if (C > 1) cluster.sync();
     }
   }
-  // tree topology to shared memory (independent loads, one round trip)
+  // tree topology and local poses to shared memory (independent loads, one
+  // round trip: a level below then waits for shared memory only)
   for (int i = tid; i < P; i += kRefitThreads) {
     sm.parent[i] = a.stat[i].parent;
     sm.lorder[i] = a.level_order[i];
   }
   for (int i = tid; i <= a.n_levels; i += kRefitThreads) sm.lstart[i] = a.level_start[i];
+#pragma unroll 4
+  for (int k = tid; k < P * 12; k += kRefitThreads) sm.world[k] = local[k];
   __syncthreads();
 
   int r;  // lane inside the part's group of four: rows 0..2, lane 3 helps with the FP32 bounds
   const int q = quad_item(tid, r);
   const unsigned int qmask = 0xFu << (lane & ~3);
 
-  // 1. compose, level by level (parents are on earlier levels); lane r
-  //    computes row r of W_i = W_parent o L_i
-  for (int L = 0; L < a.n_levels; ++L) {
+  // 1. compose in place, level by level (parents are on earlier levels): a
+  //    root's world pose is its local one, and lane r computes row r of
+  //    W_i = W_parent o L_i once the group has read all of L_i
+  for (int L = 1; L < a.n_levels; ++L) {
     const int b = sm.lstart[L], e = sm.lstart[L + 1];
     for (int j = b + q; j < e; j += kQuadsPerPass) {
-      if (r == 3) continue;
       const int i = sm.lorder[j];
-      const int p = sm.parent[i];
-      const double *Li = local + 12 * i;
+      double *Wi = sm.world + 12 * i;
+      const double *Wp = sm.world + 12 * sm.parent[i] + 4 * (r < 3 ? r : 2);
+      const double p0 = Wp[0], p1 = Wp[1], p2 = Wp[2], p3 = Wp[3];
       double out[4];
-      if (p < 0) {
+      out[0] = p0 * Wi[0] + p1 * Wi[4] + p2 * Wi[8];
+      out[1] = p0 * Wi[1] + p1 * Wi[5] + p2 * Wi[9];
+      out[2] = p0 * Wi[2] + p1 * Wi[6] + p2 * Wi[10];
+      out[3] = p0 * Wi[3] + p1 * Wi[7] + p2 * Wi[11] + p3;
+      __syncwarp(qmask);
+      if (r < 3) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) out[c] = Li[4 * r + c];
-      } else {
-        const double *Wp = sm.world + 12 * p + 4 * r;
-        const double p0 = Wp[0], p1 = Wp[1], p2 = Wp[2], p3 = Wp[3];
-        out[0] = p0 * Li[0] + p1 * Li[4] + p2 * Li[8];
-        out[1] = p0 * Li[1] + p1 * Li[5] + p2 * Li[9];
-        out[2] = p0 * Li[2] + p1 * Li[6] + p2 * Li[10];
-        out[3] = p0 * Li[3] + p1 * Li[7] + p2 * Li[11] + p3;
+        for (int c = 0; c < 4; ++c) Wi[4 * r + c] = out[c];
       }
-#pragma unroll
-      for (int c = 0; c < 4; ++c) sm.world[12 * i + 4 * r + c] = out[c];
     }
     __syncthreads();
   }
