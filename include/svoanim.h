@@ -102,8 +102,9 @@ typedef int32_t svo_status;
 #define SVO_TRACE_WAVEFRONT 1024u /* launch shape (results unchanged): the trace runs as two launches.  The
                                      first runs every ray's first culling pass (Sec. IV-A/B), writes the
                                      miss of each ray whose part spheres are all missed and queues the
-                                     others with their candidate parts; the second traces the queued rays
-                                     only, 32 to a warp, from those candidates on.  Pays where few rays
+                                     others with their candidate parts (through the scene grid where that
+                                     pays); the second traces the queued rays only, from those
+                                     candidates on.  Pays where few rays
                                      meet a part (incoherent rays in sparse scenes), so that a warp of the
                                      fused launch descends with few lanes.  Needs CULL | SORT; not with
                                      REUSE or GRID.  The queue (64 bytes per ray of the largest launch) is
