@@ -55,6 +55,7 @@ __device__ __forceinline__ uint32_t hit_color(const uint4 h, const PartStatic *_
 __global__ void k_hit_colors(const uint4 *__restrict__ hits, unsigned long long n,
                              const PartStatic *__restrict__ stat, int n_parts, uint32_t background,
                              uint32_t *__restrict__ rgb) {
+  wait_for_previous();
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
     __stcs(&rgb[i], hit_color(__ldcs(&hits[i]), stat, n_parts, background));
@@ -181,6 +182,7 @@ __device__ __forceinline__ bool shade_fast(uint32_t color, float t, float4 o, fl
 __global__ void k_shade(const float4 *__restrict__ rays, const uint4 *__restrict__ hits, unsigned long long n,
                         const PartStatic *__restrict__ stat, const double *__restrict__ inv64, int n_parts,
                         const __grid_constant__ ShadeArgs sa, uint32_t *__restrict__ rgb) {
+  wait_for_previous();
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const uint4 h = __ldcs(&hits[i]);
@@ -210,16 +212,14 @@ unsigned int grid_for(unsigned long long n, int threads, int n_sm) {
 cudaError_t launch_hit_colors(const uint4 *hits, unsigned long long n, const PartStatic *stat, int n_parts,
                               uint32_t background, uint32_t *rgb, int n_sm, cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  k_hit_colors<<<grid_for(n, 256, n_sm), 256, 0, stream>>>(hits, n, stat, n_parts, background, rgb);
-  return cudaGetLastError();
+  return launch_after(k_hit_colors, grid_for(n, 256, n_sm), 256, 0, stream, hits, n, stat, n_parts, background, rgb);
 }
 
 cudaError_t launch_shade(const float4 *rays, const uint4 *hits, unsigned long long n, const PartStatic *stat,
                          const double *inv64, int n_parts, const ShadeArgs &sa, uint32_t *rgb, int n_sm,
                          cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  k_shade<<<grid_for(n, 256, n_sm), 256, 0, stream>>>(rays, hits, n, stat, inv64, n_parts, sa, rgb);
-  return cudaGetLastError();
+  return launch_after(k_shade, grid_for(n, 256, n_sm), 256, 0, stream, rays, hits, n, stat, inv64, n_parts, sa, rgb);
 }
 
 }  // namespace svo

@@ -37,6 +37,7 @@ __device__ __forceinline__ void cell_range(float c, float r, float lo, float inv
 }
 
 __global__ void __launch_bounds__(kGridThreads) k_build_grid(const __grid_constant__ GridLaunch L) {
+  wait_for_previous();
   const GridJob job = L.jobs[blockIdx.x];
   SceneGrid *grid = job.grid;
   if (grid->stale == 0) return;  // block-uniform
@@ -187,8 +188,7 @@ cudaError_t launch_grid(const GridLaunch &L, cudaStream_t stream) {
   const size_t smem = grid_smem_bytes(gmax);
   cudaError_t e = cudaFuncSetAttribute(k_build_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_build_grid<<<(unsigned int)L.n_jobs, kGridThreads, smem, stream>>>(L);
-  return cudaGetLastError();
+  return launch_after(k_build_grid, (unsigned int)L.n_jobs, kGridThreads, smem, stream, L);
 }
 
 }  // namespace svo

@@ -23,6 +23,7 @@ constexpr int kKeyBits = 14;  // 16384 bins: the histogram (64 KiB) stays in L1 
 constexpr int kBins = 1 << kKeyBits;
 
 __global__ void k_raygen(RaygenArgs a, float4 *__restrict__ rays) {
+  wait_for_previous();
   const unsigned long long n = (unsigned long long)a.width * a.height;
   for (unsigned long long k = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; k < n;
        k += (unsigned long long)gridDim.x * blockDim.x) {
@@ -257,8 +258,7 @@ cudaError_t launch_raygen(const RaygenArgs &a, float *rays, int n_sm, cudaStream
   unsigned long long blocks = (n + 255) / 256;
   if (blocks > (unsigned long long)n_sm * 16) blocks = (unsigned long long)n_sm * 16;
   if (blocks == 0) return cudaSuccess;
-  k_raygen<<<(unsigned int)blocks, 256, 0, stream>>>(a, reinterpret_cast<float4 *>(rays));
-  return cudaGetLastError();
+  return launch_after(k_raygen, (unsigned int)blocks, 256, 0, stream, a, reinterpret_cast<float4 *>(rays));
 }
 
 size_t order_scratch_bytes(unsigned long long n) {

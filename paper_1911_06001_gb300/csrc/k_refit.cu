@@ -146,6 +146,7 @@ __device__ __forceinline__ float norm_up(float x, float y, float z) {
 __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *local, double *keep, bool read_keep,
                                             unsigned char *refit_smem) {
   namespace cg = cooperative_groups;
+  wait_for_previous();
   const cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int P = a.n_parts;
@@ -489,12 +490,14 @@ cudaError_t launch_clusters(void (*kern)(Params...), int n, int cluster, size_t 
   cfg.blockDim = dim3(kRefitThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = (unsigned int)cluster;
-  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned int)cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 

@@ -102,14 +102,6 @@ constexpr int kListThreadsPerSM = 512;
 // 175 / 165 us a call with others behind it.
 constexpr int kImageThreadsPerSM = 512;
 
-// Programmatic dependent launches: the kernels of the chain culling -> trace
-// -> FP64 pass are launched while the one before still runs (launch_after),
-// do what does not depend on it, and wait for all of it here.  None asks for
-// its successor to start early: the successor's blocks would only wait, in
-// registers and shared memory that other streams' kernels can use (eight
-// views of three graphs at a time: 103 us a graph, 119 with early starts).
-__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 constexpr unsigned long long kRayBits = 40;
 constexpr uint32_t kNoCand = 0xFFFFFFFFu;  // a list slot without stored leaves
 
@@ -2705,22 +2697,6 @@ cudaError_t blocks_per_sm(K kern, int block, size_t smem, int &per_sm) {
   if (e != cudaSuccess) return e;
   g_occ.push_back({fn, dev, smem, per_sm});
   return cudaSuccess;
-}
-
-// Launches a kernel that waits for the one before it by itself.
-template <typename T>
-cudaError_t launch_after(void (*kern)(T), unsigned int grid, int block, size_t smem, cudaStream_t stream, const T &L) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3((unsigned int)block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, L);
 }
 
 template <int NI, int BLOCK>
