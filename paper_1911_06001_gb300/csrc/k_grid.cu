@@ -1,11 +1,14 @@
 // k_grid.cu -- the scene-level grid over the part spheres (the larger
 // structure the paper suggests for scenes of many parts, Sec. V-E).
 //
-// Built on demand: every refit marks a scene's grid stale, and a trace with
-// SVO_TRACE_GRID first launches k_build_grid, whose block for that scene
-// rebuilds the grid only if it is stale.  Scenes never traced with the grid
-// pay one store per refit.  The staleness lives on the device, so the rule
-// holds for any mix of eager launches and CUDA-graph replays.
+// Built on demand: every refit marks a scene's grid stale, and a trace that
+// may walk it first launches k_build_grid, whose block for that scene rebuilds
+// the grid only if it is stale.  Scenes never traced with the grid pay one
+// store per refit.  The state lives on the device, so the rule holds for any
+// mix of eager launches and CUDA-graph replays.  Traces of one scene may run on
+// several streams at once: of their builds the one that claims the stale grid
+// rebuilds it, the others return at once, and no trace walks it before it is
+// published as ready.
 //
 // One block per scene: the spheres' box (block reduction), per-cell counts
 // (shared-memory atomics), an exclusive scan, the fill, and a sort of each
@@ -40,7 +43,10 @@ __global__ void __launch_bounds__(kGridThreads) k_build_grid(const __grid_consta
   wait_for_previous();
   const GridJob job = L.jobs[blockIdx.x];
   SceneGrid *grid = job.grid;
-  if (grid->stale == 0) return;  // block-uniform
+  __shared__ int claimed;
+  if (threadIdx.x == 0) claimed = atomicCAS(&grid->stale, kGridStale, kGridBuilding) == kGridStale;
+  __syncthreads();
+  if (!claimed) return;
   const int tid = threadIdx.x, P = job.n_parts, G = grid->G, NC3 = G * G * G;
   int32_t *cell_start = grid->cell_start;
   int32_t *cell_parts = grid->cell_parts;
@@ -173,7 +179,11 @@ __global__ void __launch_bounds__(kGridThreads) k_build_grid(const __grid_consta
     }
     grid->valid = fits ? 1 : 0;
     grid->sparse = gcnt_total <= kGridSparse * NC3 ? 1 : 0;
-    grid->stale = 0;
+  }
+  __syncthreads();  // every thread's part of the lists is written
+  if (tid == 0) {
+    __threadfence();
+    atomicExch(&grid->stale, kGridReady);
   }
 }
 

@@ -442,7 +442,7 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
   }
   // the scene grid, if any, no longer matches the spheres: the next grid
   // trace rebuilds it first
-  if (a.grid != nullptr && gtid == 0) a.grid->stale = 1;
+  if (a.grid != nullptr && gtid == 0) a.grid->stale = kGridStale;
 }
 
 template <bool INLINE, int CAP>

@@ -750,6 +750,14 @@ __device__ __forceinline__ void list_insert(float (&ct)[kCap], float (&ce)[kCap]
   }
 }
 
+// Whether a grid may be walked: once it is ready, what its build wrote is
+// visible to the caller, and it stays as it is until the scene's next refit.
+__device__ __forceinline__ bool grid_ready(const SceneGrid *g) {
+  int state;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(state) : "l"(&g->stale) : "memory");
+  return state == kGridReady;
+}
+
 // Where a ray enters the scene grid: its first cell (cur), the step along
 // each axis, 1/d (rd), the crossing of the cell's far plane per axis (tn) and
 // the end of its segment in the grid's box (t1).  Returns whether it walks;
@@ -816,8 +824,8 @@ __device__ __forceinline__ bool grid_enter(const RayW &r, const SceneGrid &g, in
 // then the lanes descend their candidates together, in order of entry, so
 // that the warp runs the descents side by side as on the cluster level.
 template <bool STATS, int BLOCK>
-__device__ __forceinline__ bool grid_walk(const RayW &r, bool go, const SceneGrid &g,
-                                          const int32_t *__restrict__ cstart, const int32_t *__restrict__ cparts,
+__device__ __forceinline__ bool grid_walk(const RayW &r, bool go, const SceneGrid &g, const int32_t *cstart,
+                                          const int32_t *cparts,
                                           const PartHot *__restrict__ hot, const PartAux *__restrict__ aux,
                                           const Tables *tab, uint32_t stop, int top_levels, uint2 *stk, uint32_t *mbox,
                                           int mwords, CertState &st, Contenders &con, unsigned int &err,
@@ -1167,7 +1175,7 @@ __device__ void trace_ray_f32(const RayW &r, bool active, uint32_t flags, int P,
                               unsigned int &err,
                               Counters &cnt,
                               bool reuse, uint32_t prev_part, const uint8_t *__restrict__ dirty, bool &reused,
-                              const SceneGrid *__restrict__ grid, uint32_t *mbox, int mwords, uint32_t tile_words,
+                              const SceneGrid *grid, uint32_t *mbox, int mwords, uint32_t tile_words,
                               uint32_t tile_count) {
   reused = false;
   st.lo1 = st.hi1 = st.te1 = st.lo2 = st.hi_min = Num<float>::inf();
@@ -1555,6 +1563,7 @@ __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? 
   uint32_t n_rays = 0, n_flag = 0;
   const int lane = threadIdx.x & 31;
   const unsigned long long n_tiles = LIST ? (unsigned long long)*L.tile_count : L.n_tiles;
+  const SceneGrid *ready = nullptr;  // the grid this warp last found ready
   for (;;) {
     unsigned long long tile = 0;
     if (lane == 0) tile = atomicAdd(L.tile_counter, 1ull);
@@ -1574,6 +1583,11 @@ __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? 
     const PartAux *aux = staged ? sAux : I.aux;
     const Cluster *cls = staged ? sCl : I.clusters;
     const int32_t *ord = staged ? sOrd : I.order;
+    const SceneGrid *grid = nullptr;  // warp-uniform
+    if (GRID && I.grid != nullptr) {
+      if (ready != I.grid && __all_sync(0xffffffffu, grid_ready(I.grid))) ready = I.grid;
+      if (ready == I.grid) grid = ready;
+    }
     const int rpl = L.rays_per_lane;
 #pragma unroll 1
     for (int j = 0; j < rpl; ++j) {
@@ -1589,7 +1603,7 @@ __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? 
       bool reused;
       trace_ray_f32<STATS, BLOCK, GRID, LIST>(r, active, L.flags, P, NC, hot, aux, cls, ord, tab, sTopAddr,
                                               (TOP && ntop_all > 0) ? L.top_levels : 0, sStack, st, con,
-                                              err, cnt, reuse, prev_part, I.dirty, reused, GRID ? I.grid : nullptr,
+                                              err, cnt, reuse, prev_part, I.dirty, reused, grid,
                                               sMbox, L.mbox_words, words, count);
       finish_ray<NI, STATS>(L, I, it, ray, in_range, reused, r, aux, st, con, lane, err, cnt, n_flag);
     }
@@ -1633,12 +1647,19 @@ __host__ __device__ inline size_t cull_smem_bytes(int max_parts, int max_cells) 
          (size_t)(max_cells + 1 + (max_cells & 1 ? 0 : 1) + kGridSparse * max_cells) * sizeof(uint16_t);
 }
 
+// Called by the whole block; usable: the block's shared word for its verdict
+// on the grid, which other streams' builds may be about to change.
 template <int NI, bool STATS>
-__device__ __forceinline__ CullTables cull_stage(const TraceItem &I, unsigned char *smem, GridDims *dims) {
+__device__ __forceinline__ CullTables cull_stage(const TraceItem &I, unsigned char *smem, GridDims *dims, int *usable) {
   float4 *sphere = reinterpret_cast<float4 *>(smem);
   CullTables t;
   const SceneGrid *g = STATS ? nullptr : I.grid;
-  t.grid = g != nullptr && g->valid != 0 && g->sparse != 0 ? g : nullptr;
+  if (g != nullptr) {
+    if (threadIdx.x == 0) *usable = grid_ready(g) && g->valid != 0 && g->sparse != 0;
+    __syncthreads();
+    if (!*usable) g = nullptr;
+  }
+  t.grid = g;
   const float4 *src = t.grid ? I.sphere : I.sph;
   for (int i = threadIdx.x; i < I.n_parts; i += kCullThreads) sphere[i] = src[i];
   uint16_t *cstart = reinterpret_cast<uint16_t *>(sphere + I.n_parts), *cparts = cstart;
@@ -1763,6 +1784,7 @@ __global__ void __launch_bounds__(kCullThreads, kCullThreadsPerSM / kCullThreads
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned long long sChunk;
   __shared__ unsigned int sNext;
+  __shared__ int sUsable;
   __shared__ GridDims sDims;
   // [per-warp rings of member-test pairs | tables]
   int2 *ring = reinterpret_cast<int2 *>(smem) + (threadIdx.x >> 5) * kPackRing;
@@ -1774,7 +1796,7 @@ __global__ void __launch_bounds__(kCullThreads, kCullThreadsPerSM / kCullThreads
   int staged = -1;
   CullTables t = {nullptr, nullptr, nullptr, nullptr, nullptr};
   if (L.same_scene && L.n_items == 1) {
-    t = cull_stage<NI, STATS>(L.items[0], tables, &sDims);
+    t = cull_stage<NI, STATS>(L.items[0], tables, &sDims, &sUsable);
     __syncthreads();
     // every warp claims its tiles for itself, one at a time while the counter keeps up (one claim a ns)
     const unsigned long long run = L.n_tiles <= 65536ull ? 1ull : 4ull;
@@ -1805,7 +1827,7 @@ __global__ void __launch_bounds__(kCullThreads, kCullThreadsPerSM / kCullThreads
         const unsigned long long stop = min(last, it + 1 < L.n_items ? L.items[it + 1].tile_begin : L.n_tiles);
         __syncthreads();  // every warp is done with the last tables and the last counter
         if (threadIdx.x == 0) sNext = 0;
-        if (it != staged) t = cull_stage<NI, STATS>(I, tables, &sDims);
+        if (it != staged) t = cull_stage<NI, STATS>(I, tables, &sDims, &sUsable);
         staged = it;
         __syncthreads();
         const auto claim = [&](unsigned long long &tile, unsigned long long &end) {

@@ -914,7 +914,7 @@ svo_status scene_create(svo_ctx *ctx, int32_t n_parts, const svo_handle *asset, 
     SceneGrid g = {};
     g.G = grid_G;
     g.cap = grid_cap;
-    g.stale = 1;
+    g.stale = kGridStale;
     g.cell_start = s->d_cell_start;
     g.cell_parts = s->d_cell_parts;
     e = cudaMemcpy(s->d_grid, &g, sizeof(g), cudaMemcpyHostToDevice);

@@ -84,11 +84,17 @@ struct SceneGrid {
   int32_t G;        // cells per axis
   int32_t valid;    // 0: the lists overflowed or the grid is too far from the origin: trace by clusters
   int32_t cap;      // capacity of cell_parts
-  int32_t stale;    // 1: a refit changed the spheres since the last build
+  int32_t stale;    // kGridReady, kGridStale or kGridBuilding
   int32_t sparse;   // 1: at most kGridSparse entries per cell on average
   int32_t *cell_start;  // G^3 + 1
   int32_t *cell_parts;
 };
+// States of a scene's grid.  A refit makes it stale; the one build launch that
+// takes it from stale to building rebuilds it and publishes it as ready.  Only a
+// ready grid is walked (grid_ready, k_trace.cu): a trace that finds it building
+// -- another stream's trace of the same scene has begun to -- goes by the
+// clusters, so streams neither share a half-written grid nor wait for one another.
+constexpr int kGridReady = 0, kGridStale = 1, kGridBuilding = 2;
 constexpr int kGridMinParts = 16;      // scenes from this size on get a grid
 constexpr int kGridWalkMinParts = 64;  // and from this one on SVO_TRACE_GRID walks it
 constexpr int kGridSparse = 2;
