@@ -1562,7 +1562,7 @@ __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? 
   Counters cnt = {0, 0, 0, 0, 0, 0, 0, 0};
   uint32_t n_rays = 0, n_flag = 0;
   const int lane = threadIdx.x & 31;
-  const unsigned long long n_tiles = LIST ? (unsigned long long)*L.tile_count : L.n_tiles;
+  const unsigned long long n_tiles = LIST ? min((unsigned long long)*L.tile_count, L.n_tiles) : L.n_tiles;
   const SceneGrid *ready = nullptr;  // the grid this warp last found ready
   for (;;) {
     unsigned long long tile = 0;
@@ -1715,8 +1715,10 @@ __device__ __forceinline__ void cull_finish(const TraceLaunchT<NI> &L, const Tra
     unsigned int base = 0;
     if (lane == leader) base = atomicAdd(&L.queue_count[it], (unsigned int)__popc(m));
     base = __shfl_sync(0xffffffffu, base, leader);
-    if (queued) {
-      QueueEntry *q = L.queue + I.qbase + base + (unsigned int)__popc(m & ((1u << lane) - 1u));
+    const unsigned long long at = base + (unsigned long long)__popc(m & ((1u << lane) - 1u));
+    if (queued && at >= I.n) atomicOr(L.err, kErrShared);  // another launch counted here as well
+    if (queued && at < I.n) {
+      QueueEntry *q = L.queue + I.qbase + at;
       q->id = make_uint4((uint32_t)ray, (uint32_t)(ray >> 32), __float_as_uint(over_t), 0u);
       q->ct = make_float4(ct[0], ct[1], ct[2], ct[3]);
       q->ce = make_float4(ce[0], ce[1], ce[2], ce[3]);
@@ -1980,6 +1982,10 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_cull(const __grid_constan
     unsigned int slot = 0;
     if (lane == 0) slot = atomicAdd(L.tile_count, 1u);
     slot = __shfl_sync(0xffffffffu, slot, 0);
+    if (slot >= L.n_tiles) {  // another launch counted here as well
+      if (lane == 0) atomicOr(L.err, kErrShared);
+      continue;
+    }
     if (lane < 16) {
       uint32_t w = (uint32_t)tile;
       if (lane == 1) w = (open || cnt > (uint32_t)kTileParts) ? kTileOpen : cnt;
@@ -2657,10 +2663,11 @@ __global__ void __launch_bounds__(kBlock) k_fix(const __grid_constant__ TraceLau
     }
     __shared__ bool last;
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&L.clean[kCounterWords - 1], 1ull) == gridDim.x - 1;
+    if (threadIdx.x == 0)  // counts the blocks and wraps to zero with the last
+      last = atomicInc(reinterpret_cast<unsigned int *>(&L.clean[kCounterWords - 1]), gridDim.x - 1) == gridDim.x - 1;
     __syncthreads();
     if (last)
-      for (int k = threadIdx.x; k < (int)kCounterWords; k += kBlock) L.clean[k] = 0ull;
+      for (int k = threadIdx.x; k < (int)kCounterWords - 1; k += kBlock) L.clean[k] = 0ull;
   }
   // count fixed rays once per launch
   if (L.stats && blockIdx.x == 0 && threadIdx.x == 0 && (L.flags & SVO_TRACE_STATS)) atomicAdd(&L.stats->fixed, n);

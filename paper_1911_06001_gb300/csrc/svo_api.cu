@@ -100,7 +100,8 @@ struct Slot {
   // counter of the wavefront descent launch, then kMaxBatchItems 32-bit queue counts and the FP64 pass's
   // blocks done.  Two sets.  The first is at zero between calls: a call that runs the FP64 pass has it
   // cleared there, any other clears it at its end.  The second belongs to a deferred FP64 pass, which reads
-  // it later, and is cleared at the start of each such call.
+  // it later, and is cleared at the start of each such call.  (The blocks done wrap to zero by themselves:
+  // should two launches ever share a slot at the same time, the state is whole again once both are done.)
   unsigned long long *d_counters = nullptr;
   bool counters_lost = false;  // a launch failed half-way: the first set is cleared before the next call
   unsigned long long *d_fix = nullptr;
@@ -176,13 +177,31 @@ AssetRec *find_asset(svo_ctx *ctx, svo_handle h) {
   return a->live ? a : nullptr;
 }
 
+bool capturing(cudaStream_t stream) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(stream, &c) != cudaSuccess || c != cudaStreamCaptureStatusNone;
+}
+
+// Zeroes a stream's new launch counters: on that stream, or -- while it is being captured, when
+// a memset there is only recorded, for a replay that may come after other calls -- now.
+cudaError_t clear_counters(unsigned long long *counters, size_t bytes, cudaStream_t stream) {
+  if (!capturing(stream)) return cudaMemsetAsync(counters, 0, bytes, stream);
+  cudaStream_t own = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(counters, 0, bytes, own);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(own);
+  cudaStreamDestroy(own);
+  return e;
+}
+
 svo_status get_slot(svo_ctx *ctx, void *stream, unsigned long long need, Slot **out) {
   std::lock_guard<std::mutex> g(ctx->mu);
   Slot &s = ctx->slots[stream];
   if (!s.d_counters) {
     unsigned long long *p = nullptr;
     CK(cudaMalloc(&p, 2 * kCounterWords * sizeof(unsigned long long)));
-    const cudaError_t e = cudaMemsetAsync(p, 0, 2 * kCounterWords * sizeof(unsigned long long), (cudaStream_t)stream);
+    const cudaError_t e = clear_counters(p, 2 * kCounterWords * sizeof(unsigned long long), (cudaStream_t)stream);
     if (e != cudaSuccess) {
       cudaFree(p);
       return fail(SVO_ERR_CUDA, "launch counters: %s", cudaGetErrorString(e));
@@ -477,7 +496,8 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
   L.clean = fix && !defer ? counters : nullptr;
   if (defer || slot->counters_lost) {
     CK(cudaMemsetAsync(counters, 0, kCounterWords * sizeof(unsigned long long), st));
-    if (!defer) slot->counters_lost = false;
+    // a recorded memset clears them for its replays only
+    if (!defer && !capturing(st)) slot->counters_lost = false;
   }
   // the scene grids this launch walks: SVO_TRACE_GRID's from
   // kGridWalkMinParts parts on, and those its culling launch uses
@@ -695,9 +715,9 @@ svo_status svo_check_device(svo_ctx *ctx) {
   CK(cudaMemcpy(&e, ctx->d_err, sizeof(e), cudaMemcpyDeviceToHost));
   CK(cudaMemset(ctx->d_err, 0, sizeof(unsigned int)));
   if (e == 0) return ok();
-  return fail(SVO_ERR_DEVICE, "device checks failed: 0x%x%s%s%s%s", e, (e & kErrNodeIndex) ? " node-index" : "",
+  return fail(SVO_ERR_DEVICE, "device checks failed: 0x%x%s%s%s%s%s", e, (e & kErrNodeIndex) ? " node-index" : "",
               (e & kErrFixOverflow) ? " fix-list-overflow" : "", (e & kErrSingular) ? " singular-pose" : "",
-              (e & kErrStack) ? " stack" : "");
+              (e & kErrStack) ? " stack" : "", (e & kErrShared) ? " scratch-shared" : "");
 }
 
 svo_status svo_build_host(const svo_desc *d, uint64_t *n_nodes, uint64_t *n_leaves, void *nodes, uint32_t *rgb) {

@@ -26,6 +26,7 @@ constexpr unsigned int kErrNodeIndex = 1u;      // a child index fell outside th
 constexpr unsigned int kErrFixOverflow = 2u;    // the FP64 re-intersection list overflowed
 constexpr unsigned int kErrSingular = 4u;       // a composed pose was not invertible
 constexpr unsigned int kErrStack = 8u;          // traversal stack exceeded kMaxDepth
+constexpr unsigned int kErrShared = 16u;        // a queue of the launch counted more than it can hold: its scratch was in use twice
 
 // Static per-part data written at scene_create.
 struct PartStatic {
