@@ -381,29 +381,7 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
     if (e == cudaSuccess) slot->queue_cap = total_rays;
     return e;
   };
-  // Rays said to be worth sorting by origin are traced in the wavefront shape
-  // instead (results are the same): its culling launch needs no order, and its
-  // lanes refill.  Should more than half the rays meet a part, the descent launch
-  // stands back for the single launch, in the given order (gate).  Per trace,
-  // sorted against this: 2.1 M incoherent rays and 128 parts 878 -> 461 us, 1 M
-  // inside 1024 parts 1397 -> 556, 100 K and 200 parts 152 -> 137, 1 M close rays
-  // of which three quarters hit 2100 -> 2010, a coherent 1920x1080 image
-  // 326 -> 323.  By direction alone sorting stays: it brings shuffled camera rays
-  // back into order, which serves them better.  Without room for the queue the
-  // rays are sorted.
-  L.gate = 0;
-  if (order_mode == 2 && !wave && L.n_items == 1 && !(L.flags & (SVO_TRACE_REUSE | SVO_TRACE_GRID | SVO_TRACE_STATS)) &&
-      (L.flags & (SVO_TRACE_CULL | SVO_TRACE_SORT)) == (SVO_TRACE_CULL | SVO_TRACE_SORT)) {
-    if (grow_queue() == cudaSuccess) {
-      wave = true;
-      order_mode = 0;
-      L.flags |= SVO_TRACE_WAVEFRONT;
-      L.gate = total_rays / 2 + 1;
-    } else {
-      cudaGetLastError();
-    }
-  }
-  if (order_mode) {
+  if (order_mode) {  // also where the rays are then not sorted: one call at full size makes room for every route
     size_t need = 0;
     for (int i = 0; i < L.n_items; ++i) need += (order_scratch_bytes(L.items[i].n) + 255) & ~size_t(255);
     if (need > slot->order_cap) {
@@ -418,6 +396,33 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
       if (e != cudaSuccess) return fail(SVO_ERR_OOM, "ray-order scratch: %s", cudaGetErrorString(e));
       slot->order_cap = need;
     }
+  }
+  // Rays said to be worth sorting by origin are traced in the wavefront shape
+  // instead (results are the same): its culling launch needs no order, and its
+  // lanes refill.  Should more than half the rays meet a part, the descent launch
+  // stands back for the single launch, in the given order (gate).  Per trace,
+  // sorted against this: 2.1 M incoherent rays and 128 parts 878 -> 461 us, 1 M
+  // inside 1024 parts 1397 -> 556, 100 K and 200 parts 152 -> 137, 1 M close rays
+  // of which three quarters hit 2100 -> 2010, a coherent 1920x1080 image
+  // 326 -> 323.  By direction alone sorting stays: it brings shuffled camera rays
+  // back into order, which serves them better.  Without room for the queue, or
+  // where a stream being captured would have to grow it, the rays are sorted.
+  L.gate = 0;
+  if (order_mode == 2 && !wave && L.n_items == 1 && !(L.flags & (SVO_TRACE_REUSE | SVO_TRACE_GRID | SVO_TRACE_STATS)) &&
+      (L.flags & (SVO_TRACE_CULL | SVO_TRACE_SORT)) == (SVO_TRACE_CULL | SVO_TRACE_SORT)) {
+    bool room = total_rays <= slot->queue_cap;
+    if (!room && !capturing(st)) {
+      room = grow_queue() == cudaSuccess;
+      if (!room) cudaGetLastError();
+    }
+    if (room) {
+      wave = true;
+      order_mode = 0;
+      L.flags |= SVO_TRACE_WAVEFRONT;
+      L.gate = total_rays / 2 + 1;
+    }
+  }
+  if (order_mode) {
     size_t off = 0;
     if (L.n_items == 1) {
       uint32_t *perm = nullptr;
