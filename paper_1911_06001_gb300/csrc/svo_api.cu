@@ -121,6 +121,7 @@ struct Slot {
   size_t order_cap = 0;
   QueueEntry *d_queue = nullptr;             // SVO_TRACE_WAVEFRONT: the ray queue
   unsigned long long queue_cap = 0;          // entries
+  unsigned long long queue_refused = ~0ull;  // a queue of this size found no room: ORDER_ORIGIN no longer asks for it
 };
 
 }  // namespace
@@ -411,9 +412,15 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
   if (order_mode == 2 && !wave && L.n_items == 1 && !(L.flags & (SVO_TRACE_REUSE | SVO_TRACE_GRID | SVO_TRACE_STATS)) &&
       (L.flags & (SVO_TRACE_CULL | SVO_TRACE_SORT)) == (SVO_TRACE_CULL | SVO_TRACE_SORT)) {
     bool room = total_rays <= slot->queue_cap;
-    if (!room && !capturing(st)) {
-      room = grow_queue() == cudaSuccess;
-      if (!room) cudaGetLastError();
+    if (!room && total_rays < slot->queue_refused && !capturing(st)) {
+      const cudaError_t e = grow_queue();
+      room = e == cudaSuccess;
+      if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();  // not an error of this call
+        slot->queue_refused = total_rays;
+      } else if (e != cudaSuccess) {
+        return fail(SVO_ERR_CUDA, "ray queue: %s", cudaGetErrorString(e));
+      }
     }
     if (room) {
       wave = true;
