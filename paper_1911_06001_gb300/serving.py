@@ -32,13 +32,19 @@ from dataclasses import dataclass, field
 
 import numpy as np
 
-from . import TRACE_DEFAULT, TRACE_STATS, Context, trace_image
+from . import TRACE_DEFAULT, TRACE_ORDER_ORIGIN, TRACE_STATS, TRACE_WAVEFRONT, Context, trace_image
 
 RAY_BYTES = 32
 HIT_BYTES = 16
 # per-ray scratch the library keeps per stream (FP64 list and pool offsets, the FP64 pass's
-# leaf pool of 3 entries of 16 B per ray, ray ordering)
-SCRATCH_BYTES_PER_RAY = 8 + 4 + 48 + 10
+# leaf pool of 3 entries of 16 B per ray, image tile entries, ray ordering)
+SCRATCH_BYTES_PER_RAY = 8 + 4 + 48 + 4 + 10
+QUEUE_BYTES_PER_RAY = 64  # the ray queue of the wavefront shape
+
+
+def scratch_bytes_per_ray(flags: int) -> int:
+    """Scratch per ray of traces with these flags (rays to be ordered by origin may take the wavefront shape)."""
+    return SCRATCH_BYTES_PER_RAY + (QUEUE_BYTES_PER_RAY if flags & (TRACE_WAVEFRONT | TRACE_ORDER_ORIGIN) else 0)
 
 
 class AdmissionError(RuntimeError):
@@ -175,7 +181,7 @@ class Server:
             rays = torch.empty((max_batch_rays, 8), dtype=torch.float32, device=self.dev)
             hits = torch.empty((max_batch_rays, 2), dtype=torch.int64, device=self.dev)
             self.slots.append(_Slot(st, rays, hits, max_batch_rays))
-        per_ray = RAY_BYTES + HIT_BYTES + SCRATCH_BYTES_PER_RAY
+        per_ray = RAY_BYTES + HIT_BYTES + scratch_bytes_per_ray(self.flags)
         self.budget = memory_budget if memory_budget is not None else n_slots * max_batch_rays * per_ray
         self.per_ray = per_ray
         self.queue = RequestQueue(max_batch_rays, self.budget, per_ray, max_wait)
