@@ -109,7 +109,7 @@ struct Slot {
   uint4 *d_cand = nullptr;                   // pool of leaves stored for the FP64 pass
   unsigned long long cand_cap = 0;           // pool entries (kPoolPerRay per ray of capacity)
   uint32_t *d_off = nullptr;                 // per list slot: its first pool entry
-  TileEntry *d_tiles = nullptr;              // image tiles to trace (tile_capacity(cap) entries)
+  TileEntry *d_tiles = nullptr;              // image tiles to trace (tile_capacity(cap) entries; may be missing)
   TraceLaunch *pending = nullptr;            // launch whose FP64 pass is deferred
   char *d_stage = nullptr;                   // trace_rays_host: two halves of rays | hits | flags
   cudaStream_t pipe[3] = {nullptr, nullptr, nullptr};  // trace_rays_host: copy in, trace, copy out
@@ -235,12 +235,22 @@ svo_status get_slot(svo_ctx *ctx, void *stream, unsigned long long need, Slot **
     cudaError_t e = cudaMalloc(&p, cap * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc(&c, ccap * sizeof(uint4));
     if (e == cudaSuccess) e = cudaMalloc(&o, cap * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&s.d_tiles, tile_capacity(cap) * sizeof(TileEntry));
     if (e != cudaSuccess) {
       if (p) cudaFree(p);
       if (c) cudaFree(c);
       if (o) cudaFree(o);
       return fail(SVO_ERR_OOM, "scratch for %llu rays: %s", cap, cudaGetErrorString(e));
+    }
+    // without room for these, image traces run in one launch
+    e = cudaMalloc(&s.d_tiles, tile_capacity(cap) * sizeof(TileEntry));
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();  // not an error of this call
+      s.d_tiles = nullptr;
+    } else if (e != cudaSuccess) {
+      cudaFree(p);
+      cudaFree(c);
+      cudaFree(o);
+      return fail(SVO_ERR_CUDA, "image tile entries: %s", cudaGetErrorString(e));
     }
     s.d_fix = p;
     s.cap = cap;
