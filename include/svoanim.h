@@ -81,10 +81,12 @@ typedef int32_t svo_status;
 #define SVO_TRACE_DEFER_FIX 16u /* with FP64_FIX: collect flagged rays but leave the FP64 pass to
                                    trace_fix_pending (lets a caller time the two passes apart) */
 #define SVO_TRACE_ORDER_DIR 32u    /* trace rays in an order grouped by direction (results unchanged) */
-#define SVO_TRACE_ORDER_ORIGIN 64u /* ... grouped by origin cell, then direction (results unchanged) */
+#define SVO_TRACE_ORDER_ORIGIN 64u /* ... grouped by origin cell, then direction (results unchanged); one
+                                      scene's rays take a faster shape where there is one (trace_rays) */
 #define SVO_TRACE_IMAGE_TILES 128u /* rays are the pixels of a row-major image whose width is in bits
                                       16..31 of flags: warps take 8 x 4 pixel tiles instead of 32
-                                      consecutive rays (results unchanged; ignored with ORDER_*) */
+                                      consecutive rays (results unchanged; ignored where the rays are
+                                      sorted) */
 #define SVO_TRACE_IMAGE(width) (SVO_TRACE_IMAGE_TILES | ((uint32_t)(width) << 16))
 #define SVO_TRACE_GRID 512u  /* cull through the scene-level grid (scenes of 64+ parts, built by every
                                 refit; Sec. V-E): each ray walks the grid cells it crosses front to back,
@@ -337,9 +339,13 @@ svo_status trace_rays(svo_scene *scene, const float *rays, uint64_t n, svo_hit *
                       uint32_t flags, svo_trace_stats *stats, void *stream);
 /* (With SVO_TRACE_ORDER_DIR / _ORIGIN the rays are first counting-sorted by a
  * 14-bit direction / origin-cell key into per-stream scratch, grown like the
- * FP64 list; hits still land at each ray's own index.  trace_rays with _ORIGIN
- * takes the wavefront shape instead where its flags allow it, with that
- * shape's queue as scratch, and sorts where the queue finds no room.) */
+ * FP64 list; hits still land at each ray's own index.  Where a trace_rays call,
+ * or a batch of one item, with _ORIGIN and CULL | SORT is faster without the sort
+ * -- not with REUSE, GRID or STATS -- it is traced in the wavefront shape or in
+ * the given order instead, chosen by the number of rays and parts and by how many
+ * of a sample of the rays meet a part.  Its scratch is the sort's and, for 128
+ * parts or 2^18 rays and more, the wavefront shape's queue; without room for the
+ * queue the rays are sorted.) */
 /* Batched trace: every item's rays against its own scene, in one persistent
  * launch whose thread blocks take fixed-size tiles of rays from a device work
  * counter (async), or -- with SVO_TRACE_WAVEFRONT -- in a culling launch and a

@@ -41,6 +41,7 @@ __device__ __forceinline__ void cell_range(float c, float r, float lo, float inv
 
 __global__ void __launch_bounds__(kGridThreads) k_build_grid(const __grid_constant__ GridLaunch L) {
   wait_for_previous();
+  if (L.cond != nullptr && (*L.cond < L.cond_min || *L.cond >= L.cond_max)) return;  // not walked by this trace
   const GridJob job = L.jobs[blockIdx.x];
   SceneGrid *grid = job.grid;
   __shared__ int claimed;

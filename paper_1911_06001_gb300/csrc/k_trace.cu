@@ -75,7 +75,8 @@ struct TraceLaunchT {
   unsigned long long *queue_tile;   // SVO_TRACE_WAVEFRONT: tile counter of the descent launch
   TileEntry *tiles;                 // tile-culled image trace: the tiles to trace
   unsigned int *tile_count;         // their number
-  unsigned long long gate;          // see TraceLaunch
+  unsigned int *gate_count;         // see TraceLaunch
+  unsigned int gate;
   unsigned long long *clean;        // the FP64 pass leaves these kCounterWords at zero, and every dirty flag (nullptr: no)
 };
 
@@ -1535,7 +1536,7 @@ __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? 
   const uint32_t sTopAddr = (uint32_t)__cvta_generic_to_shared(sTop);
   load_tables(tab);
   wait_for_previous();
-  if (L.gate && *L.queue_count < L.gate) return;  // the descent launch has the queued rays
+  if (L.gate && *L.gate_count < L.gate) return;  // the wavefront shape's launches have the rays
   if (L.one_scene) {
     const TraceItem &I0 = L.items[0];
     for (int i = threadIdx.x; i < I0.n_parts; i += BLOCK) {
@@ -1795,6 +1796,7 @@ __global__ void __launch_bounds__(kCullThreads, kCullThreadsPerSM / kCullThreads
   uint32_t n_rays = 0;
   const int lane = threadIdx.x & 31;
   wait_for_previous();
+  if (L.gate && *L.gate_count >= L.gate) return;  // the single launch traces every ray
   int staged = -1;
   CullTables t = {nullptr, nullptr, nullptr, nullptr, nullptr};
   if (L.same_scene && L.n_items == 1) {
@@ -1850,6 +1852,27 @@ __global__ void __launch_bounds__(kCullThreads, kCullThreadsPerSM / kCullThreads
     }
   }
   if (STATS) flush_stats(L.stats, cnt, n_rays, 0u);
+}
+
+// How many of kSampleRays rays, spread evenly over the item's, meet a part
+// sphere: one warp a ray, its lanes over the parts.  A few us for fewer than
+// 128 parts, against the culling launch's 60 to 120 on a million rays, which
+// told the same but was thrown away where most rays meet a part.
+__global__ void __launch_bounds__(256) k_sample(const __grid_constant__ TraceLaunchT<1> L) {
+  const TraceItem &I = L.items[0];
+  const int lane = threadIdx.x & 31;
+  const unsigned int warp = blockIdx.x * 8u + (threadIdx.x >> 5);
+  wait_for_previous();
+  RayW r;
+  const bool active = load_ray(I, I.n * warp / kSampleRays, true, r);
+  bool met = false;
+  for (int p = lane; p < I.n_parts && active; p += 32) {
+    float tin, tref;
+    met = met || sphere_cull(r, I.sph[p], tin, tref);
+  }
+  met = __any_sync(0xffffffffu, met);
+  const int n = __syncthreads_count(lane == 0 && met);
+  if (threadIdx.x == 0) atomicAdd(L.gate_count, (unsigned int)n);
 }
 
 // The tile-culling launch of an image trace.  One warp takes one 8x4-pixel
@@ -2024,7 +2047,7 @@ __global__ void __launch_bounds__(BLOCK, 512 / BLOCK) k_descend(const __grid_con
   int32_t *sOrd = reinterpret_cast<int32_t *>(sCl + sc);
   load_tables(tab);
   wait_for_previous();
-  if (L.gate && *L.queue_count >= L.gate) return;  // the single launch traces every ray
+  if (L.gate && *L.gate_count >= L.gate) return;  // the single launch traces every ray
   if (L.one_scene) {
     const TraceItem &I0 = L.items[0];
     for (int i = threadIdx.x; i < I0.n_parts; i += BLOCK) {
@@ -2771,12 +2794,10 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
     e = launch_after(kq, (unsigned int)(n_sm * per_sm), BLOCK, smem, stream, L);
     if constexpr (NI == 1) {
       if (e != cudaSuccess || !L.gate) return e;
-      TraceLaunchT<NI> G = L;
-      G.tile_counter = L.queue_tile;  // the culling launch has used the other, and only one of these two claims from it
       auto kg = k_trace<NI, false, BLOCK, false, false>;
       e = blocks_per_sm(kg, BLOCK, smem, per_sm);
       if (e != cudaSuccess) return e;
-      return launch_after(kg, (unsigned int)(n_sm * (per_sm < 1 ? 1 : per_sm)), BLOCK, smem, stream, G);
+      return launch_after(kg, (unsigned int)(n_sm * (per_sm < 1 ? 1 : per_sm)), BLOCK, smem, stream, L);
     }
     return e;
   }
@@ -2883,6 +2904,7 @@ void fill_launch(const TraceLaunch &src, TraceLaunchT<NI> &dst) {
   dst.queue_tile = src.queue_tile;
   dst.tiles = src.tiles;
   dst.tile_count = src.tile_count;
+  dst.gate_count = src.gate_count;
   dst.gate = src.gate;
   dst.clean = src.clean;
 }
@@ -2912,6 +2934,12 @@ cudaError_t launch_trace(const TraceLaunch &L, int n_sm, cudaStream_t stream) {
   TraceLaunchT<kMaxBatchItems> &p = batch_params();
   fill_launch(L, p);
   return launch_trace_t(p, n_sm, stream);
+}
+
+cudaError_t launch_sample(const TraceLaunch &L, cudaStream_t stream) {
+  TraceLaunchT<1> l1;
+  fill_launch(L, l1);
+  return launch_after(k_sample, kSampleRays / 8, 256, 0, stream, l1);
 }
 
 cudaError_t launch_fix(const TraceLaunch &L, int n_sm, cudaStream_t stream) {

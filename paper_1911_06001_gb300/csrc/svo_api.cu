@@ -85,6 +85,25 @@ inline size_t stage_half_bytes(unsigned long long n) { return ((size_t)n * (32 +
 // against the clusters.
 constexpr unsigned long long kCullGridTests = 1ull << 25, kCullGridRays = 32;
 
+// A one-scene call with ORDER_ORIGIN takes one of two shapes with the same
+// results; the sort by origin that the flag first stood for is no longer one of
+// them.  Random rays and shuffled camera rays, hit or not, 100 K to 2 M against 1
+// to 1024 parts (484 calls): none is slower than with the sort before, which took
+// 1.37 (16 parts) to 1.7 (1, 1024) times as long on average.
+// From kOrderWaveParts parts on: the wavefront shape.  Sorted, with the same
+// descent, against it:
+//   128 parts, 1 M rays, few hit 813 / 629 us, all hit 689 / 781
+//   1024 parts, 1 M rays, few hit 1729 / 998, all hit 1707 / 1033
+// Below: the single launch in the given order, but for many rays few of which
+// meet a part.  That is told from kSampleRays rays tested in a launch of their own
+// (k_sample) and decided on the device: past the share 3/8 + parts/205 the
+// wavefront shape's launches stand back.  Given order / wavefront, 1 M rays:
+//   16 parts: 28% hit 294 / 272, 52% 355 / 377     32: 30% 396 / 352, 55% 459 / 469
+//   64 parts: 56% hit 520 / 492, 78% 558 / 598     128: 78% 734 / 655, all 764 / 758
+//   100 K rays, 64 parts: none hit 92 / 110, all 102 / 140
+constexpr int kOrderWaveParts = 128;
+constexpr unsigned long long kOrderWaveRays = 1ull << 18;
+
 constexpr unsigned long long kTileCullMin = 256;
 constexpr int kTileCullParts = 20;
 
@@ -96,7 +115,8 @@ inline unsigned long long tile_capacity(unsigned long long cap) { return cap / 1
 
 // Scratch of one stream: launch counters and the FP64 re-intersection list.
 struct Slot {
-  // [0] tile counter, [1] fix count and queued image tiles (32 bits each), [2] pool count, [3] tile
+  // [0] tile counter, [1] fix count and queued image tiles (32 bits each), [2] pool count and sampled rays
+  // that meet a part (likewise), [3] tile
   // counter of the wavefront descent launch, then kMaxBatchItems 32-bit queue counts and the FP64 pass's
   // blocks done.  Two sets.  The first is at zero between calls: a call that runs the FP64 pass has it
   // cleared there, any other clears it at its end.  The second belongs to a deferred FP64 pass, which reads
@@ -408,35 +428,34 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
       slot->order_cap = need;
     }
   }
-  // Rays said to be worth sorting by origin are traced in the wavefront shape
-  // instead (results are the same): its culling launch needs no order, and its
-  // lanes refill.  Should more than half the rays meet a part, the descent launch
-  // stands back for the single launch, in the given order (gate).  Per trace,
-  // sorted against this: 2.1 M incoherent rays and 128 parts 878 -> 461 us, 1 M
-  // inside 1024 parts 1397 -> 556, 100 K and 200 parts 152 -> 137, 1 M close rays
-  // of which three quarters hit 2100 -> 2010, a coherent 1920x1080 image
-  // 326 -> 323.  By direction alone sorting stays: it brings shuffled camera rays
-  // back into order, which serves them better.  Without room for the queue, or
-  // where a stream being captured would have to grow it, the rays are sorted.
+  // Rays said to be worth sorting by origin (see kOrderWaveParts).  Without room
+  // for the queue, or where a stream being captured would have to grow it, they
+  // are sorted.
   L.gate = 0;
+  L.gate_count = reinterpret_cast<unsigned int *>(counters + 2) + 1;
   if (order_mode == 2 && !wave && L.n_items == 1 && !(L.flags & (SVO_TRACE_REUSE | SVO_TRACE_GRID | SVO_TRACE_STATS)) &&
       (L.flags & (SVO_TRACE_CULL | SVO_TRACE_SORT)) == (SVO_TRACE_CULL | SVO_TRACE_SORT)) {
-    bool room = total_rays <= slot->queue_cap;
-    if (!room && total_rays < slot->queue_refused && !capturing(st)) {
-      const cudaError_t e = grow_queue();
-      room = e == cudaSuccess;
-      if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();  // not an error of this call
-        slot->queue_refused = total_rays;
-      } else if (e != cudaSuccess) {
-        return fail(SVO_ERR_CUDA, "ray queue: %s", cudaGetErrorString(e));
-      }
-    }
-    if (room) {
-      wave = true;
+    const int parts = L.items[0].n_parts;
+    if (parts < kOrderWaveParts && total_rays < kOrderWaveRays) {
       order_mode = 0;
-      L.flags |= SVO_TRACE_WAVEFRONT;
-      L.gate = total_rays / 2 + 1;
+    } else {
+      bool room = total_rays <= slot->queue_cap;
+      if (!room && total_rays < slot->queue_refused && !capturing(st)) {
+        const cudaError_t e = grow_queue();
+        room = e == cudaSuccess;
+        if (e == cudaErrorMemoryAllocation) {
+          cudaGetLastError();  // not an error of this call
+          slot->queue_refused = total_rays;
+        } else if (e != cudaSuccess) {
+          return fail(SVO_ERR_CUDA, "ray queue: %s", cudaGetErrorString(e));
+        }
+      }
+      if (room) {
+        wave = true;
+        order_mode = 0;
+        L.flags |= SVO_TRACE_WAVEFRONT;
+        if (parts < kOrderWaveParts) L.gate = kSampleRays * 3 / 8 + 5 * (unsigned int)parts;
+      }
     }
   }
   if (order_mode) {
@@ -533,7 +552,9 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
       it.grid = nullptr;
   }
   if (((L.flags & SVO_TRACE_GRID) && !L.tiles) || wave) {
+    if (L.gate) CK(launch_sample(L, st));
     GridLaunch gl;
+    if (L.gate) gl.cond = L.gate_count, gl.cond_max = L.gate;
     if (grid_jobs(L.items, L.n_items, gl) > 0) CK(launch_grid(gl, st));
   }
   cudaError_t e = launch_trace(L, ctx->n_sm, st);

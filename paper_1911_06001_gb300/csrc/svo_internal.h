@@ -208,7 +208,8 @@ struct TraceLaunch {
   unsigned long long *queue_tile;     // SVO_TRACE_WAVEFRONT: tile counter of the descent launch; zeroed
   TileEntry *tiles;                   // tile-culled image trace: the tiles to trace (nullptr: one launch over all)
   unsigned int *tile_count;           // their number; zeroed
-  unsigned long long gate;            // wavefront: from this many queued rays on the single launch traces them all (0: never)
+  unsigned int *gate_count;           // of kSampleRays rays, those that meet a part (k_sample); zeroed
+  unsigned int gate;                  // wavefront: from this many of them on the single launch traces the rays (0: never)
   unsigned long long *clean;          // counters the FP64 pass leaves at zero, with every dirty flag (nullptr: no)
 };
 
@@ -241,6 +242,9 @@ inline cudaError_t launch_after(void (*kern)(Params...), unsigned int grid, int 
 // Kernel launchers (k_trace.cu, k_refit.cu).
 cudaError_t launch_trace(const TraceLaunch &L, int n_sm, cudaStream_t stream);
 cudaError_t launch_fix(const TraceLaunch &L, int n_sm, cudaStream_t stream);
+// Counts in *L.gate_count the rays of a sample of the one item's that meet a part.
+constexpr unsigned int kSampleRays = 1024;
+cudaError_t launch_sample(const TraceLaunch &L, cudaStream_t stream);
 
 // Leaf colours of n hits (k_color.cu); see trace_hit_colors.
 cudaError_t launch_hit_colors(const uint4 *hits, unsigned long long n, const PartStatic *stat, int n_parts,
@@ -322,6 +326,10 @@ struct GridJob {
 struct GridLaunch {
   GridJob jobs[kMaxBatchItems];
   int32_t n_jobs;
+  // build only if cond_min <= *cond < cond_max (nullptr: always): whether the trace will walk the
+  // grids may be decided on the device
+  const unsigned int *cond = nullptr;
+  unsigned int cond_min = 0, cond_max = 0;
 };
 size_t grid_smem_bytes(int G);
 cudaError_t launch_grid(const GridLaunch &L, cudaStream_t stream);

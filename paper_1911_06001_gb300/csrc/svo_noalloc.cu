@@ -149,6 +149,7 @@ extern "C" svo_status trace_rays_noalloc(svo_scene *s, const float *rays, uint64
   L->tile_count = nullptr;
   L->clean = nullptr;  // cleared below
   L->gate = 0;
+  L->gate_count = nullptr;
   // clear what the kernels expect at zero: the tile counter, the list count and the pool count
   e = cudaMemsetAsync(base, 0, 3 * sizeof(unsigned long long), st);
   if (e == cudaSuccess && (flags & SVO_TRACE_GRID)) {
