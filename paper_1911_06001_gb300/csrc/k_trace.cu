@@ -1194,7 +1194,7 @@ __device__ void trace_ray_f32(const RayW &r, bool active, uint32_t flags, int P,
     float last_t = -Num<float>::inf();
     int last_p = -1;
     bool need = active;
-    if (GRID && grid != nullptr && grid->valid != 0) {  // warp-uniform: one item per warp
+    if (GRID && grid != nullptr && grid->valid != 0) {  // warp-uniform: one item per warp, one tile's list
       // a ray the walk cannot take safely goes on to the cluster level below
       const SceneGrid &g = *grid;
       const bool walked = grid_walk<STATS, BLOCK>(r, need, g, g.cell_start, g.cell_parts, hot, aux, tab, stop,
@@ -1516,7 +1516,8 @@ __device__ __forceinline__ void finish_ray(const TraceLaunchT<NI> &L, const Trac
 // TOP: the top levels of every part staged in shared memory (a separate
 // instantiation: the staged-node base is one more live register, which the
 // common kernel does not carry).
-// LIST: only the image tiles k_tile_cull queued, each with its parts.
+// LIST: only the image tiles k_tile_cull queued, each with its parts; with GRID
+// the tiles without a list walk the grid.
 // IMAGE: every item's rays are image tiles (the same code at more registers).
 template <int NI, bool STATS, int BLOCK, bool REUSE, bool GRID, bool TOP = false, bool LIST = false, bool IMAGE = false>
 __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? kListThreadsPerSM : IMAGE ? kImageThreadsPerSM : kTraceThreadsPerSM) / BLOCK) k_trace(const __grid_constant__ TraceLaunchT<NI> L) {
@@ -1585,7 +1586,7 @@ __global__ void __launch_bounds__(BLOCK, (STATS || REUSE || GRID ? 512 : LIST ? 
     const Cluster *cls = staged ? sCl : I.clusters;
     const int32_t *ord = staged ? sOrd : I.order;
     const SceneGrid *grid = nullptr;  // warp-uniform
-    if (GRID && I.grid != nullptr) {
+    if (GRID && I.grid != nullptr && (!LIST || count == kTileOpen)) {
       if (ready != I.grid && __all_sync(0xffffffffu, grid_ready(I.grid))) ready = I.grid;
       if (ready == I.grid) grid = ready;
     }
@@ -2002,6 +2003,8 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_cull(const __grid_constan
       }
       continue;
     }
+    const bool listed = !open && cnt <= (uint32_t)kTileParts;
+    if (!listed && lane == 0 && (L.flags & SVO_TRACE_GRID) && I.grid != nullptr) *L.gate_count = 1u;
     unsigned int slot = 0;
     if (lane == 0) slot = atomicAdd(L.tile_count, 1u);
     slot = __shfl_sync(0xffffffffu, slot, 0);
@@ -2011,7 +2014,7 @@ __global__ void __launch_bounds__(kTileThreads) k_tile_cull(const __grid_constan
     }
     if (lane < 16) {
       uint32_t w = (uint32_t)tile;
-      if (lane == 1) w = (open || cnt > (uint32_t)kTileParts) ? kTileOpen : cnt;
+      if (lane == 1) w = listed ? cnt : kTileOpen;
       if (lane >= 2) w = reinterpret_cast<const uint32_t *>(list)[lane - 2];
       reinterpret_cast<uint32_t *>(L.tiles + slot)[lane] = w;
     }
@@ -2752,7 +2755,7 @@ cudaError_t blocks_per_sm(K kern, int block, size_t smem, int &per_sm) {
 }
 
 template <int NI, int BLOCK>
-cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t stream) {
+cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, const GridLaunch *tile_grids, int n_sm, cudaStream_t stream) {
   const bool stats = (L.flags & SVO_TRACE_STATS) && L.stats;
   const bool reuse = (L.flags & SVO_TRACE_REUSE) != 0;
   bool walk = (L.flags & SVO_TRACE_GRID) != 0 && !reuse;
@@ -2812,10 +2815,15 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
     if (grid == 0) return cudaSuccess;
     e = launch_after(k_tile_cull<NI>, (unsigned int)grid, kTileThreads, 0, stream, L);
     if (e != cudaSuccess) return e;
+    if (tile_grids) {
+      e = launch_grid(*tile_grids, stream);
+      if (e != cudaSuccess) return e;
+    }
     const size_t smem = trace_smem_bytes(L.stack_levels, L.one_scene ? L.items[0].n_parts : 0,
-                                         L.one_scene ? L.items[0].n_clusters : 0, BLOCK, 0, 0);
-    auto kl = reuse ? k_trace<NI, false, BLOCK, true, false, false, true>
-                    : k_trace<NI, false, BLOCK, false, false, false, true>;
+                                         L.one_scene ? L.items[0].n_clusters : 0, BLOCK, walk ? L.mbox_words : 0, 0);
+    auto kl = reuse  ? k_trace<NI, false, BLOCK, true, false, false, true>
+              : walk ? k_trace<NI, false, BLOCK, false, true, false, true>
+                     : k_trace<NI, false, BLOCK, false, false, false, true>;
     e = blocks_per_sm(kl, BLOCK, smem, per_sm);
     if (e != cudaSuccess) return e;
     grid = (unsigned long long)n_sm * (per_sm < 1 ? 1 : per_sm);
@@ -2850,10 +2858,10 @@ cudaError_t launch_trace_b(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t str
 }
 
 template <int NI>
-cudaError_t launch_trace_t(const TraceLaunchT<NI> &L, int n_sm, cudaStream_t stream) {
-  if (L.block == 64) return launch_trace_b<NI, 64>(L, n_sm, stream);
-  if (L.block == 256) return launch_trace_b<NI, 256>(L, n_sm, stream);
-  return launch_trace_b<NI, 128>(L, n_sm, stream);
+cudaError_t launch_trace_t(const TraceLaunchT<NI> &L, const GridLaunch *tile_grids, int n_sm, cudaStream_t stream) {
+  if (L.block == 64) return launch_trace_b<NI, 64>(L, tile_grids, n_sm, stream);
+  if (L.block == 256) return launch_trace_b<NI, 256>(L, tile_grids, n_sm, stream);
+  return launch_trace_b<NI, 128>(L, tile_grids, n_sm, stream);
 }
 
 // Four blocks, the most that fit: an entry is a chain of dependent reads and
@@ -2925,15 +2933,15 @@ TraceLaunchT<kMaxBatchItems> &batch_params() {
   return *p;
 }
 
-cudaError_t launch_trace(const TraceLaunch &L, int n_sm, cudaStream_t stream) {
+cudaError_t launch_trace(const TraceLaunch &L, const GridLaunch *tile_grids, int n_sm, cudaStream_t stream) {
   if (L.n_items <= 1) {
     TraceLaunchT<1> l1;
     fill_launch(L, l1);
-    return launch_trace_t(l1, n_sm, stream);
+    return launch_trace_t(l1, tile_grids, n_sm, stream);
   }
   TraceLaunchT<kMaxBatchItems> &p = batch_params();
   fill_launch(L, p);
-  return launch_trace_t(p, n_sm, stream);
+  return launch_trace_t(p, tile_grids, n_sm, stream);
 }
 
 cudaError_t launch_sample(const TraceLaunch &L, cudaStream_t stream) {

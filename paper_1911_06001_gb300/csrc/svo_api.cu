@@ -493,7 +493,10 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
   // the counting build, staged top levels and wider tiles, for a scene-grid
   // trace with items that are not images, and for rays read over the host
   // link (the tiles that go on would be read twice: 250,000 mapped rays take
-  // 201 us in one launch, 221 in two).
+  // 201 us in one launch, 221 in two).  With SVO_TRACE_GRID a tile without a
+  // part list walks the grid, which is built only if there is one: 1000 touching
+  // parts, 640x360 from outside / from close 323 / 946 us by the clusters, 179 /
+  // 497 by the grid (198 / 528 with every tile walking it).
   L.tiles = nullptr;
   L.tile_count = reinterpret_cast<unsigned int *>(counters + 1) + 1;
   if (!wave && !host_rays && ctx->rays_per_lane == 1 && ctx->smem_levels == 0 && !(L.flags & SVO_TRACE_STATS) &&
@@ -551,13 +554,15 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
                                    : !cull_grids || it.n < kCullGridRays * (unsigned long long)it.n_parts)
       it.grid = nullptr;
   }
-  if (((L.flags & SVO_TRACE_GRID) && !L.tiles) || wave) {
-    if (L.gate) CK(launch_sample(L, st));
-    GridLaunch gl;
-    if (L.gate) gl.cond = L.gate_count, gl.cond_max = L.gate;
-    if (grid_jobs(L.items, L.n_items, gl) > 0) CK(launch_grid(gl, st));
+  GridLaunch gl;
+  const bool grids = ((L.flags & SVO_TRACE_GRID) || wave) && grid_jobs(L.items, L.n_items, gl) > 0;
+  if (L.gate) {
+    CK(launch_sample(L, st));
+    gl.cond = L.gate_count, gl.cond_max = L.gate;
   }
-  cudaError_t e = launch_trace(L, ctx->n_sm, st);
+  if (L.tiles) gl.cond = L.gate_count, gl.cond_min = 1, gl.cond_max = ~0u;
+  if (grids && !L.tiles) CK(launch_grid(gl, st));
+  cudaError_t e = launch_trace(L, grids && L.tiles ? &gl : nullptr, ctx->n_sm, st);
   delete slot->pending;
   slot->pending = nullptr;
   if (L.clean) {

@@ -208,7 +208,8 @@ struct TraceLaunch {
   unsigned long long *queue_tile;     // SVO_TRACE_WAVEFRONT: tile counter of the descent launch; zeroed
   TileEntry *tiles;                   // tile-culled image trace: the tiles to trace (nullptr: one launch over all)
   unsigned int *tile_count;           // their number; zeroed
-  unsigned int *gate_count;           // of kSampleRays rays, those that meet a part (k_sample); zeroed
+  unsigned int *gate_count;           // of kSampleRays rays, those that meet a part (k_sample), or
+                                      // SVO_TRACE_GRID by image tiles: whether a tile walks a grid; zeroed
   unsigned int gate;                  // wavefront: from this many of them on the single launch traces the rays (0: never)
   unsigned long long *clean;          // counters the FP64 pass leaves at zero, with every dirty flag (nullptr: no)
 };
@@ -240,7 +241,9 @@ inline cudaError_t launch_after(void (*kern)(Params...), unsigned int grid, int 
 #endif
 
 // Kernel launchers (k_trace.cu, k_refit.cu).
-cudaError_t launch_trace(const TraceLaunch &L, int n_sm, cudaStream_t stream);
+struct GridLaunch;
+// tile_grids: the grid build to launch between the culling of image tiles and their trace, or nullptr.
+cudaError_t launch_trace(const TraceLaunch &L, const GridLaunch *tile_grids, int n_sm, cudaStream_t stream);
 cudaError_t launch_fix(const TraceLaunch &L, int n_sm, cudaStream_t stream);
 // Counts in *L.gate_count the rays of a sample of the one item's that meet a part.
 constexpr unsigned int kSampleRays = 1024;
