@@ -116,19 +116,37 @@ __device__ __forceinline__ uint32_t shade_channel_fast(uint32_t c, float s, bool
   return f >= 255.f ? 255u : (uint32_t)f;
 }
 
+// An upper bound of |x| in FP32 from its high word (FP64 instructions are what
+// bounds this kernel), clamped to [2^-126, 2^127]: the bounds below are then
+// decided by their other terms, or fail.
+__device__ __forceinline__ float mag_up(double x) {
+  const int h = min(max(__double2hiint(x) & 0x7fffffff, 897 << 20), (1150 << 20) - 1);
+  return __int_as_float((h - (896 << 20) + 1) << 3);
+}
+
 // The same decisions taken in FP32 wherever their error cannot change them.
 // The ray is moved to its hit's t in FP64, so that what FP32 compares are the
 // distances from the leaf's planes, leaves in size: u_k with an error of 2^-24
-// of (|u_k| + size), tau_k = u_k / d'_k within e_k below (its last
-// term: the FP64 transforms' own rounding, of the exact way too).  Returns false where
-// the entry face, the test for a start inside the leaf or a channel's rounding
-// is too close to call.
+// of (|u_k| + size), tau_k = u_k / d'_k within e_k below.  To that comes the FP64
+// rounding of both ways: of the origin's transform, a chain of up to five
+// operations on terms of at most mo that may cancel (a part far from the world's
+// origin, a small part), 5 + 3 units of 2^-53 mo, and of the direction's, 4 + 3
+// units of md for each t moved along it.  Where eleven units of them (1.2e-15) are
+// more than 2^-24 of (|u_k| + size) the exact way is taken.  n_ainv: the inverse's
+// infinity norm, rounded up.  Returns false there, and where the entry face, the
+// test for a start inside the leaf or a channel's rounding is too close to call.
 __device__ __forceinline__ bool shade_fast(uint32_t color, float t, float4 o, float4 d, const double *__restrict__ m,
-                                           int D, unsigned long long vox, const ShadeArgs &sa, uint32_t &out) {
+                                           float n_ainv, int D, unsigned long long vox, const ShadeArgs &sa,
+                                           uint32_t &out) {
   constexpr float kU32 = 5.9604644775390625e-8f;  // 2^-24
   const uint32_t mask = (1u << D) - 1u;
   const double size64 = __longlong_as_double((long long)(1023 - D) << 52);
   const float size = __int_as_float((127 - D) << 23);
+  const float md = n_ainv * fmaxf(fmaxf(fabsf(d.x), fabsf(d.y)), fabsf(d.z));
+  const float mo = fmaf(n_ainv, fmaxf(fmaxf(fabsf(o.x), fabsf(o.y)), fabsf(o.z)),
+                        fmaxf(fmaxf(mag_up(m[3]), mag_up(m[7])), mag_up(m[11])));
+  if (!(1.2e-15f * (2.0f + fmaf(fabsf(t), md, mo)) <= kU32 * size)) return false;
+  const float dmin = fmaxf(1e-20f, 2.1e-8f * md);  // 1.2e-15 |tau| md <= 2^-24 |u| from here on
   const double ox = o.x, oy = o.y, oz = o.z, dx = d.x, dy = d.y, dz = d.z, th = t;
   float best = -__int_as_float(0x7f800000), err = 0.f, next = best, next_err = 0.f;
   int kf = -1;
@@ -141,8 +159,8 @@ __device__ __forceinline__ bool shade_fast(uint32_t color, float t, float4 o, fl
     const float u0 = (float)(lo - fma(th, dl, ol)), dk = (float)dl;
     const float u = dk > 0.f ? u0 : u0 + size;
     const float inv = __frcp_rn(dk);
-    const float tau = u * inv, e = fmaf(8.0f * kU32, fabsf(u) + size, 4e-15f * (2.0f + fabsf(t * dk))) * fabsf(inv);
-    sure = sure && fabsf(dk) > 1e-20f && fabsf(dk) < 1e20f;  // a zero or extreme component: the exact way
+    const float tau = u * inv, e = 10.0f * kU32 * (fabsf(u) + size) * fabsf(inv);
+    sure = sure && fabsf(dk) > dmin && fabsf(dk) < 1e20f;  // a zero or extreme component: the exact way
     if (tau > best) {
       if (best + err > next + next_err) {
         next = best;
@@ -180,8 +198,8 @@ __device__ __forceinline__ bool shade_fast(uint32_t color, float t, float4 o, fl
 // (two matrix products, three divisions, a square root and a channel each
 // about seven instructions) 0.16 M hits of 0.98 M pixels took 57 us, now 28.
 __global__ void k_shade(const float4 *__restrict__ rays, const uint4 *__restrict__ hits, unsigned long long n,
-                        const PartStatic *__restrict__ stat, const double *__restrict__ inv64, int n_parts,
-                        const __grid_constant__ ShadeArgs sa, uint32_t *__restrict__ rgb) {
+                        const PartStatic *__restrict__ stat, const PartAux *__restrict__ aux,
+                        const double *__restrict__ inv64, int n_parts, const __grid_constant__ ShadeArgs sa, uint32_t *__restrict__ rgb) {
   wait_for_previous();
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -193,7 +211,7 @@ __global__ void k_shade(const float4 *__restrict__ rays, const uint4 *__restrict
       const unsigned long long vox = ((unsigned long long)h.w << 32) | h.z;
       const int D = stat[h.y].depth;
       uint32_t lit;
-      if (!shade_fast(out, __uint_as_float(h.x), o, d, m, D, vox, sa, lit))
+      if (!shade_fast(out, __uint_as_float(h.x), o, d, m, aux[h.y].n_ainv, D, vox, sa, lit))
         lit = shade_exact(out, o, d, m, D, vox, sa);
       out = lit;
     }
@@ -216,10 +234,10 @@ cudaError_t launch_hit_colors(const uint4 *hits, unsigned long long n, const Par
 }
 
 cudaError_t launch_shade(const float4 *rays, const uint4 *hits, unsigned long long n, const PartStatic *stat,
-                         const double *inv64, int n_parts, const ShadeArgs &sa, uint32_t *rgb, int n_sm,
+                         const PartAux *aux, const double *inv64, int n_parts, const ShadeArgs &sa, uint32_t *rgb, int n_sm,
                          cudaStream_t stream) {
   if (n == 0) return cudaSuccess;
-  return launch_after(k_shade, grid_for(n, 256, n_sm), 256, 0, stream, rays, hits, n, stat, inv64, n_parts, sa, rgb);
+  return launch_after(k_shade, grid_for(n, 256, n_sm), 256, 0, stream, rays, hits, n, stat, aux, inv64, n_parts, sa, rgb);
 }
 
 }  // namespace svo

@@ -1435,7 +1435,7 @@ svo_status trace_shade(svo_scene *s, const float *rays, const svo_hit *hits, uin
   if (reinterpret_cast<uintptr_t>(rgb) & 3) return fail(SVO_ERR_ARG, "trace_shade: rgb not 4-byte aligned");
   CK(cudaSetDevice(s->ctx->device));
   CK(launch_shade(reinterpret_cast<const float4 *>(rays), reinterpret_cast<const uint4 *>(hits), n, s->d_stat,
-                  s->d_inv64, s->P, sa, rgb, s->ctx->n_sm, (cudaStream_t)stream));
+                  s->d_aux, s->d_inv64, s->P, sa, rgb, s->ctx->n_sm, (cudaStream_t)stream));
   return ok();
 }
 

@@ -260,7 +260,7 @@ struct ShadeArgs {
   uint32_t background;
 };
 cudaError_t launch_shade(const float4 *rays, const uint4 *hits, unsigned long long n, const PartStatic *stat,
-                         const double *inv64, int n_parts, const ShadeArgs &sa, uint32_t *rgb, int n_sm,
+                         const PartAux *aux, const double *inv64, int n_parts, const ShadeArgs &sa, uint32_t *rgb, int n_sm,
                          cudaStream_t stream);
 
 struct RaygenArgs {
