@@ -476,9 +476,20 @@ __global__ void __launch_bounds__(kRefitThreads) k_refit_batch(const __grid_cons
 // the cluster: 1024 parts 153 -> 52 us (4 blocks: 72), 128 parts 25.6 -> 19.1,
 // 64 scenes of up to 256 parts in one launch 42 -> 27 (32 parts a block: 53,
 // the launch then waits for room for its clusters).
-int refit_cluster(int n_parts) {
+//
+// Many large scenes in one launch get smaller clusters, so that every block has
+// an SM to itself: two blocks on one SM share its FP64 pipes, and clusters that
+// find no room wait for a whole round.  n_full: the scenes the launch would hold
+// if all were as large as its largest.  Per launch, clusters of 1 / 2 / 4 / 8:
+//   1024 parts, 12 scenes 425 / 315 / 260 / 240 us, 16: 426 / 316 / 259 / 465,
+//               64: 432 / 320 / 517 / 1158
+//   512 parts,  12 scenes 198 / 159 / 139 / 138,    32: 198 / 158 / 140 / 183,
+//               64: 200 / 160 / 184 / 358
+//   256 parts,  32 scenes  93 /  79 /  72 / 109,    64:  94 /  80 / 100 / 165
+int refit_cluster(int n_parts, int n_full) {
   int c = 1;
   while (c < kMaxRefitCluster && 64 * c < n_parts) c *= 2;
+  while (c > 2 && n_full > (c > 4 ? 12 : 32)) c /= 2;
   return c;
 }
 
@@ -508,7 +519,7 @@ cudaError_t launch_refit_t(const RefitArgs &a, const double *host_local, size_t 
     for (int k = 0; k < a.n_parts * 12; ++k) p.local[k] = host_local[k];
   cudaError_t e = cudaFuncSetAttribute(k_refit<INLINE, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_clusters(k_refit<INLINE, CAP>, 1, refit_cluster(a.n_parts), smem, stream, a, p);
+  return launch_clusters(k_refit<INLINE, CAP>, 1, refit_cluster(a.n_parts, 1), smem, stream, a, p);
 }
 
 }  // namespace
@@ -530,9 +541,12 @@ cudaError_t launch_refit_batch(const RefitArgs *args, const double *const *src, 
     smem = m > smem ? m : smem;
   }
   B.n = n;
-  int parts = 0;
-  for (int i = 0; i < n; ++i) parts = std::max(parts, (int)args[i].n_parts);
-  B.cluster = refit_cluster(parts);
+  int parts = 1, total = 0;
+  for (int i = 0; i < n; ++i) {
+    parts = std::max(parts, (int)args[i].n_parts);
+    total += args[i].n_parts;
+  }
+  B.cluster = refit_cluster(parts, (total + parts - 1) / parts);
   // the shared-memory attribute only ever grows: set it when this launch needs more (per device)
   constexpr int kMaxDevices = 64;
   static std::mutex mu;
