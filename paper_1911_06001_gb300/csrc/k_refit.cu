@@ -164,8 +164,8 @@ __device__ __forceinline__ void refit_scene(const RefitArgs &a, const double *lo
   if (keep) {
     for (int k = gtid; k < P * 12; k += gthreads) keep[k] = local[k];
     if (read_keep) {
-      local = keep;  // visible to the block after the barrier below
-      if (C > 1) cluster.sync();
+      local = keep;
+      sync();  // the copy below reads what other threads wrote
     }
   }
   // tree topology and local poses to shared memory (independent loads, one
