@@ -88,12 +88,15 @@ typedef int32_t svo_status;
                                       consecutive rays (results unchanged; ignored where the rays are
                                       sorted) */
 #define SVO_TRACE_IMAGE(width) (SVO_TRACE_IMAGE_TILES | ((uint32_t)(width) << 16))
-#define SVO_TRACE_GRID 512u  /* cull through the scene-level grid (scenes of 64+ parts, built by every
-                                refit; Sec. V-E): each ray walks the grid cells it crosses front to back,
-                                tests the parts listed there once each, descends them as found and stops
-                                once the next cell starts beyond its best hit.  Needs CULL | SORT; not
-                                with REUSE.  Falls back to the cluster level for smaller scenes or when
-                                the grid's lists overflowed (results are the same either way). */
+#define SVO_TRACE_GRID 512u  /* cull through the scene-level grid (scenes of 64+ parts, built by the first
+                                trace that needs it after a refit; Sec. V-E): each ray walks the grid cells
+                                it crosses front to back, tests the parts listed there once each, descends
+                                them as found and stops once the next cell starts beyond its best hit.
+                                Needs CULL | SORT; not with REUSE.  Falls back to the cluster level for
+                                smaller scenes, when the grid's lists overflowed, or while another stream's
+                                trace is building the scene's grid (results are the same either way).  Of
+                                large images (SVO_TRACE_IMAGE_TILES) whole pixel tiles are culled first, and
+                                only tiles that meet many parts walk the grid. */
 #define SVO_TRACE_REUSE 256u /* hit buffer reuse (Sec. IV-C, Fig. 5): the hits buffer holds this scene's
                                 result for the same rays from the scene's previous trace (a static
                                 camera); a ray whose intersected part spheres (at most 4) all belong to
@@ -295,8 +298,8 @@ svo_status scene_set_transforms_trs(svo_scene *scene, const double *rts_15, void
  * Sec. IV-A) and rebuild the cluster level of the sphere hierarchy.  A
  * singular pose sets the device error word (svo_check_device). */
 svo_status scene_refit(svo_scene *scene, void *stream);
-/* scene_refit of n scenes of one context in one launch, a thread block per
- * scene (async; Sec. III, Eq. 3, Sec. IV-A as scene_refit).  Each scene's
+/* scene_refit of n scenes of one context in one launch, a thread block -- above
+ * 64 parts a cluster of up to eight -- per scene (async; Sec. III, Eq. 3, Sec. IV-A as scene_refit).  Each scene's
  * refit is the same as scene_refit's, so the results are identical; the
  * batch runs the scenes side by side on the GPU instead of one launch after
  * another, for a frame that poses many scenes (a server's batch of

@@ -152,7 +152,7 @@ class Context:
         _lib.check(self.lib.trace_batch(self.h, arr, len(items), int(flags), _ptr(stats), _stream_ptr(stream)))
 
     def refit_batch(self, scenes, local_dev=None, stream=None) -> None:
-        """scene_refit of several scenes in one launch (a block per scene).
+        """scene_refit of several scenes in one launch (a block or a cluster of blocks per scene).
         local_dev: None, or one entry per scene, each None or a CUDA float64
         tensor of that scene's [P, 12] local poses."""
         n = len(scenes)

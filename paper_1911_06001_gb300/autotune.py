@@ -5,11 +5,13 @@ Knobs that change only speed, never results: the trace kernel's block size
 8), the number of top octree levels each block stages in shared memory (0-4,
 for traces of one scene), the claim order of image tiles (row by row or
 centre-out), the ray order (as given, grouped by direction, grouped by origin cell
-then direction, or -- for rays that are the pixels of an image -- warp tiles
-of 8 x 4 pixels) and the culling structure: the cluster level in one launch,
+then direction -- for one scene a request that the library may serve by another
+shape --, or -- for rays that are the pixels of an image -- warp tiles of 8 x 4
+pixels) and the culling structure: the cluster level in one launch,
 the cluster level as a culling launch plus a descent launch over the rays it
 queued (SVO_TRACE_WAVEFRONT), or -- for scenes of 64 parts or more -- the
-scene grid.  ``tune`` times every combination on the caller's rays with
+scene grid (of large images only the pixel tiles that meet many parts walk it,
+so "clusters" and "grid" differ for dense scenes only).  ``tune`` times every combination on the caller's rays with
 CUDA events (L2 flushed between repetitions), keeps the fastest, and can
 remember it in a JSON cache under a caller-chosen key (for example the scene
 and ray-batch shape).  ``tune_batch`` does the same for a batch of uneven
@@ -34,7 +36,7 @@ ORDERS = {"none": 0, "dir": TRACE_ORDER_DIR, "origin": TRACE_ORDER_ORIGIN, "imag
 _ORDER_BITS = TRACE_ORDER_DIR | TRACE_ORDER_ORIGIN | TRACE_IMAGE_TILES | 0xFFFF0000
 CULLS = {"clusters": 0, "grid": TRACE_GRID, "wavefront": TRACE_WAVEFRONT}
 _CULL_BITS = TRACE_GRID | TRACE_WAVEFRONT
-GRID_MIN_PARTS = 64  # scenes from this size on carry a grid
+GRID_MIN_PARTS = 64  # scenes from this size on are walked by their grid (TRACE_GRID)
 
 
 def _time(ctx: Context, scene, rays, hits, flags: int, reps: int, flush) -> float:

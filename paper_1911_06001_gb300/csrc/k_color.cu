@@ -11,9 +11,10 @@
 //     to world space by the inverse transpose of the part's pose (so that
 //     shear and anisotropic scale keep it perpendicular to the face).
 // trace_shade combines both into a Lambert-lit 8-bit image.  Its decisions
-// (entry face, rounding of each channel) are taken in FP64, like the FP64
+// (entry face, rounding of each channel) are those of FP64, like the FP64
 // re-intersection pass, so that they match an FP64 evaluation of the same
-// rule except within rounding distance of a tie.
+// rule except within rounding distance of a tie: FP32 takes those that its
+// error bounds settle (shade_fast), FP64 the rest (shade_exact).
 #include <cuda_runtime.h>
 
 #include <cstdint>

@@ -56,7 +56,7 @@ struct TraceLaunchT {
   unsigned long long fix_capacity;
   uint4 *fix_cand;                  // pool of stored leaves (winner, contenders or re-trace cap)
   unsigned long long cand_capacity; // pool entries
-  unsigned int *cand_count;         // pool entries taken (zeroed before the launch)
+  unsigned int *cand_count;         // pool entries taken
   uint32_t *fix_off;                // per list slot: its first pool entry, or kNoCand
   svo_trace_stats *stats;
   unsigned int *err;
@@ -332,7 +332,8 @@ __device__ __forceinline__ uint2 node_at(const uint2 *__restrict__ nodes, uint32
 // sets a bit, a pop clears the bits below its level, and a plane needs no
 // conversion from integers.  A plane P (so shifted) inflated by eta along the
 // ray is crossed at P ix + lx (its lower side) or P ix + hx (its upper side),
-// lx = -((o + 1) + eta) ix, hx = -((o + 1) - eta) ix: one FMA each.
+// lx = -((o + 1) + eta) ix, hx = -((o + 1) - eta) ix, rounded outward: one FMA
+// each.
 struct Descent {
   float ix, iy, iz, lx, ly, lz, hx, hy, hz, ox, oy, oz, tmin, tmax, tshift;
   const uint2 *nodes;
@@ -1885,7 +1886,7 @@ __global__ void __launch_bounds__(256) k_sample(const __grid_constant__ TraceLau
 }
 
 // The tile-culling launch of an image trace.  One warp takes one 8x4-pixel
-// tile (statically strided, as k_cull) and bounds its rays by a cone: apex at
+// tile after another (statically strided) and bounds its rays by a cone: apex at
 // one ray's origin o0, axis a along that ray, half angle theta with
 // 2 sin(theta/2) <= chord, the largest distance of the unit directions from
 // a, and ro, the largest distance of the origins from o0.  Then its lanes test

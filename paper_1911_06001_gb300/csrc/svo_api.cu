@@ -69,16 +69,6 @@ constexpr unsigned long long kZeroCopyMaxRays = 1ull << 18;
 // rounded so that the second half starts 256-byte aligned.
 inline size_t stage_half_bytes(unsigned long long n) { return ((size_t)n * (32 + 16 + 4) + 255) & ~(size_t)255; }
 
-// An image trace culls whole tiles in a launch of their own from this many
-// tiles and parts (of its largest scene) on.  With fewer parts the culling
-// saved is less than the launch: its reads of the rays and about 2 us.
-// Measured per call, one launch against two:
-//   1 part, 1280x768 and shading      274 -> 288 us
-//   16 parts, 1280x768 / 1920x1080    173 -> 180 / 235 -> 227
-//   up to 24 parts, 8 views 301x199   118 -> 109
-//   63 parts, 128x128 (512 tiles)     216 -> 193
-//   up to 128 parts, 9 requests      1285 -> 1091
-//   1024 parts, 1920x1080 (grid)      731 -> 544
 // The culling launch walks the scene grids when rays x parts of the launch
 // reach this, and each scene's when it has this many rays a part: building
 // the grids takes 14 to 27 us, and a walk saves about 0.4 ps a ray and part
@@ -104,6 +94,22 @@ constexpr unsigned long long kCullGridTests = 1ull << 25, kCullGridRays = 32;
 constexpr int kOrderWaveParts = 128;
 constexpr unsigned long long kOrderWaveRays = 1ull << 18;
 
+// An image trace culls whole tiles in a launch of their own from this many
+// tiles and parts (of its largest scene) on.  With fewer parts the culling
+// saved is less than the launch: its reads of the rays and about 2 us.
+// Measured per call, one launch / two, a chain of parts seen close (most rays
+// near some part) and parts scattered in a box (most rays near none):
+//   1 part, 1280x768         281 / 324      47 /  54
+//   16 parts, 1280x768       164 / 166      94 /  82
+//   16 parts, 1920x1080      254 / 252     138 / 108
+//   20 parts, 1280x768       206 / 216     112 /  96
+//   24 parts, 1920x1080      301 / 310     160 / 125
+//   63 parts, 128x128        176 / 155     105 / 101
+//   64 parts, 1280x768       233 / 253     168 / 120
+//   128 parts, 1920x1080     510 / 443     338 / 200
+//   256 parts, 96x64         301 / 309     134 / 105
+// From 12 scattered parts at full HD on two launches would be faster, up to
+// about 64 close ones one launch by a few per cent: the line lies between.
 constexpr unsigned long long kTileCullMin = 256;
 constexpr int kTileCullParts = 20;
 

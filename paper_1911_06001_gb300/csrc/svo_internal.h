@@ -183,18 +183,20 @@ inline unsigned long long layout_tiles(Item *items, int n_items, int rays_per_la
   return tiles;
 }
 
+// (The launch expects its counters at zero: the FP64 pass of the call before left them so, or -- without
+// one, or with a deferred one -- a memset did.)
 struct TraceLaunch {
   TraceItem items[kMaxBatchItems];
   int32_t n_items;
   uint32_t flags;
   unsigned long long n_tiles;
-  unsigned long long *tile_counter;   // zeroed before the launch
+  unsigned long long *tile_counter;
   unsigned long long *fix_list;       // (count << 48) | (item << 40) | ray, capacity fix_capacity
-  unsigned int *fix_count;            // zeroed before the launch
+  unsigned int *fix_count;            // list entries
   unsigned long long fix_capacity;
   uint4 *fix_cand;                    // pool of the leaves stored per list slot (fix_off)
   unsigned long long cand_capacity;   // pool entries
-  unsigned int *cand_count;           // pool entries taken; zeroed before the launch
+  unsigned int *cand_count;           // pool entries taken
   uint32_t *fix_off;                  // per list slot: first pool entry, or 0xFFFFFFFF
   svo_trace_stats *stats;
   unsigned int *err;
@@ -204,12 +206,12 @@ struct TraceLaunch {
   int32_t top_nodes;      // nodes staged in shared memory per block (0: none)
   int32_t top_levels;     // the top levels of every part that are staged
   QueueEntry *queue;                  // SVO_TRACE_WAVEFRONT: entries of every item, item i from items[i].qbase
-  unsigned int *queue_count;          // SVO_TRACE_WAVEFRONT: per item, entries queued; zeroed before the launch
-  unsigned long long *queue_tile;     // SVO_TRACE_WAVEFRONT: tile counter of the descent launch; zeroed
+  unsigned int *queue_count;          // SVO_TRACE_WAVEFRONT: per item, entries queued
+  unsigned long long *queue_tile;     // SVO_TRACE_WAVEFRONT: tile counter of the descent launch
   TileEntry *tiles;                   // tile-culled image trace: the tiles to trace (nullptr: one launch over all)
-  unsigned int *tile_count;           // their number; zeroed
+  unsigned int *tile_count;           // their number
   unsigned int *gate_count;           // of kSampleRays rays, those that meet a part (k_sample), or
-                                      // SVO_TRACE_GRID by image tiles: whether a tile walks a grid; zeroed
+                                      // SVO_TRACE_GRID by image tiles: whether a tile walks a grid
   unsigned int gate;                  // wavefront: from this many of them on the single launch traces the rays (0: never)
   unsigned long long *clean;          // counters the FP64 pass leaves at zero, with every dirty flag (nullptr: no)
 };

@@ -62,7 +62,7 @@ class BatchGraph:
     the device, composes / inverts / refits every scene, and runs
     ``trace_batch`` over all items (its ray-ordering launches, the persistent
     trace kernel and the FP64 pass included).  The refits are one launch
-    (``Context.refit_batch``: a thread block per scene, each reading its
+    (``Context.refit_batch``: a block or a cluster of blocks per scene, reading its
     poses straight from the copied buffer), so they run side by side on the
     device instead of one after another.
 

@@ -269,7 +269,8 @@ class Server:
         s.start = torch.cuda.Event(enable_timing=True)
         s.start.record(s.stream)
         # every request's scene instance is posed, then all are refitted by one
-        # launch (a block per instance; a batch leases distinct instances)
+        # launch (a block or a cluster of blocks per instance; a batch leases
+        # distinct instances)
         for t in batch:
             t.instance.set_transforms(t.request.local, stream=s.stream)
         self.ctx.refit_batch([t.instance for t in batch], stream=s.stream)
