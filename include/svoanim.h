@@ -346,9 +346,9 @@ svo_status trace_rays(svo_scene *scene, const float *rays, uint64_t n, svo_hit *
  * or a batch of one item, with _ORIGIN and CULL | SORT is faster without the sort
  * -- not with REUSE, GRID or STATS -- it is traced in the wavefront shape or in
  * the given order instead, chosen by the number of rays and parts and by how many
- * of a sample of the rays meet a part.  Its scratch is the sort's and, for 128
- * parts or 2^18 rays and more, the wavefront shape's queue; without room for the
- * queue the rays are sorted.) */
+ * of a sample of the rays meet a part.  Its scratch is the sort's and the
+ * wavefront shape's queue; without room for a queue it needs the rays are
+ * sorted.) */
 /* Batched trace: every item's rays against its own scene, in one persistent
  * launch whose thread blocks take fixed-size tiles of rays from a device work
  * counter (async), or -- with SVO_TRACE_WAVEFRONT -- in a culling launch and a

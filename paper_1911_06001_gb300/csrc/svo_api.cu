@@ -442,26 +442,24 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
   if (order_mode == 2 && !wave && L.n_items == 1 && !(L.flags & (SVO_TRACE_REUSE | SVO_TRACE_GRID | SVO_TRACE_STATS)) &&
       (L.flags & (SVO_TRACE_CULL | SVO_TRACE_SORT)) == (SVO_TRACE_CULL | SVO_TRACE_SORT)) {
     const int parts = L.items[0].n_parts;
+    bool room = total_rays <= slot->queue_cap;  // grown also where this call does not use it
+    if (!room && total_rays < slot->queue_refused && !capturing(st)) {
+      const cudaError_t e = grow_queue();
+      room = e == cudaSuccess;
+      if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();  // not an error of this call
+        slot->queue_refused = total_rays;
+      } else if (e != cudaSuccess) {
+        return fail(SVO_ERR_CUDA, "ray queue: %s", cudaGetErrorString(e));
+      }
+    }
     if (parts < kOrderWaveParts && total_rays < kOrderWaveRays) {
       order_mode = 0;
-    } else {
-      bool room = total_rays <= slot->queue_cap;
-      if (!room && total_rays < slot->queue_refused && !capturing(st)) {
-        const cudaError_t e = grow_queue();
-        room = e == cudaSuccess;
-        if (e == cudaErrorMemoryAllocation) {
-          cudaGetLastError();  // not an error of this call
-          slot->queue_refused = total_rays;
-        } else if (e != cudaSuccess) {
-          return fail(SVO_ERR_CUDA, "ray queue: %s", cudaGetErrorString(e));
-        }
-      }
-      if (room) {
-        wave = true;
-        order_mode = 0;
-        L.flags |= SVO_TRACE_WAVEFRONT;
-        if (parts < kOrderWaveParts) L.gate = kSampleRays * 3 / 8 + 5 * (unsigned int)parts;
-      }
+    } else if (room) {
+      wave = true;
+      order_mode = 0;
+      L.flags |= SVO_TRACE_WAVEFRONT;
+      if (parts < kOrderWaveParts) L.gate = kSampleRays * 3 / 8 + 5 * (unsigned int)parts;
     }
   }
   if (order_mode) {

@@ -91,3 +91,26 @@ def test_sorted_where_the_queue_has_no_room(env):
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(hits, ref)
+
+
+def test_warm_call_of_a_small_scene_serves_a_large_one(env):
+    import torch
+
+    g, ctx, scenes, rays = env
+    n = rays[0].shape[0]
+    big = ctx.scene([1] * 200, np.full(200, -1, np.int32))
+    big.set_transforms(np.array([synthetic.affine12(np.eye(3), t) for t in
+                                 np.random.default_rng(1).uniform(-9.0, 9.0, (200, 3))]))
+    big.refit()
+    stream, f = torch.cuda.Stream(), g.TRACE_DEFAULT | g.TRACE_ORDER_ORIGIN
+    ref = big.trace(rays[0])
+    hits = _hits(n)
+    torch.cuda.synchronize()
+    scenes[0].trace(rays[0], hits, flags=f, stream=stream)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    big.trace(rays[0], hits, flags=f, stream=stream)
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] == free
+    assert torch.equal(hits, ref)
+    big.close()
