@@ -560,13 +560,11 @@ svo_status run_trace(svo_ctx *ctx, TraceLaunch &L, unsigned long long total_rays
   }
   GridLaunch gl;
   const bool grids = ((L.flags & SVO_TRACE_GRID) || wave) && grid_jobs(L.items, L.n_items, gl) > 0;
-  if (L.gate) {
-    CK(launch_sample(L, st));
-    gl.cond = L.gate_count, gl.cond_max = L.gate;
-  }
+  if (L.gate) gl.cond = L.gate_count, gl.cond_max = L.gate;
   if (L.tiles) gl.cond = L.gate_count, gl.cond_min = 1, gl.cond_max = ~0u;
-  if (grids && !L.tiles) CK(launch_grid(gl, st));
-  cudaError_t e = launch_trace(L, grids && L.tiles ? &gl : nullptr, ctx->n_sm, st);
+  cudaError_t e = L.gate ? launch_sample(L, st) : cudaSuccess;  // from here on a failure leaves counters to clear
+  if (e == cudaSuccess && grids && !L.tiles) e = launch_grid(gl, st);
+  if (e == cudaSuccess) e = launch_trace(L, grids && L.tiles ? &gl : nullptr, ctx->n_sm, st);
   delete slot->pending;
   slot->pending = nullptr;
   if (L.clean) {
